@@ -10,9 +10,15 @@
 // only after the n-th was taken, its priority never exceeds the priorities before it, and a head
 // at or above every other head is taken next -- so both rules visit the pairs in the same order.
 // Each pair becomes one unique 64-bit key (~bits(p) in the high word, k*(k_max-1)+(n-2) in the
-// low word); an MSB-first radix select finds the extra-th smallest key T, and
-// n_k = 1 + #{n : key(k, n) <= T}.  The keys live in shared memory when they fit (they are
-// recomputed from the error table on every pass otherwise); no global scratch is used.
+// low word); a selection finds the extra-th smallest key T, and n_k = 1 + #{n : key(k, n) <= T}.
+// The high words live in shared memory when they fit (they are recomputed from the error table on
+// every pass otherwise); no global scratch is used.
+//
+// One CTA selects, so latency is what counts: barriers, and shared-memory atomics that meet on one
+// address.  The keys' own range is cut into 2,048 equal buckets (8-bit digits from the top, tried
+// first, put all keys into the few buckets of their common exponents: 40 us for 960 channels x 8
+// points), the bucket that holds the wanted rank is cut again if it has more than SEL_LIST keys,
+// and the rank inside it comes from counting.  960 x 8: 7.4 us; 64 x 4 keys: 9.1 -> 5.7 us.
 #include <math.h>
 
 #include "mpq_internal.cuh"
@@ -23,137 +29,161 @@ namespace mpq {
 namespace {
 
 constexpr int AB_THREADS = 1024;
-constexpr unsigned long long NO_KEY = ~0ULL;
+constexpr unsigned NO_KEY = ~0u;   // the high word of no key: a selectable p is above 0
 
-// The keys of channel k for n = 2..k_max, in n order, via callback.
+// The keys' high words of channel k for n = 2..k_max, in n order, via callback (NO_KEY: no gain).
 template <typename F>
 __device__ __forceinline__ void channel_keys(const float *__restrict__ err, int k, int k_max, F f)
 {
     const float *e = err + (size_t)k * (k_max + 1);
     float p = INFINITY;
     float prev = e[1];
+#pragma unroll 4
     for (int n = 2; n <= k_max; ++n) {
         const float cur = e[n];
         float g = __fsub_rn(prev, cur);
         if (isnan(g)) g = -INFINITY;
         p = fminf(p, g);
         prev = cur;
-        unsigned long long key = NO_KEY;
-        if (p > 0.0f) {
-            const unsigned hi = ~__float_as_uint(p);
-            const unsigned lo = (unsigned)((unsigned long long)k * (k_max - 1) + (n - 2));
-            key = ((unsigned long long)hi << 32) | lo;
-        }
-        f(n, key);
+        f(n, p > 0.0f ? ~__float_as_uint(p) : NO_KEY);
     }
 }
 
-constexpr int KEY_CACHE = 12288;   // keys held in shared memory (96 KB) when they fit
+constexpr int KEY_CACHE = 49152;   // keys' high words held in shared memory (192 KB) when they fit
+constexpr int SEL_BUCKETS = 2 * AB_THREADS;
+constexpr int SEL_LIST = AB_THREADS;
 
-// Radix select of the rank-th smallest selectable key, MSB first, 8 bits per pass.  A pass whose
-// target bucket holds one key ends the search with that key (recorded as the bucket's witness).
 // One CTA of AB_THREADS threads allocates one layer; skeys: dynamic shared memory for its keys.
 __device__ __forceinline__ void allocate_budget_cta(const float *__restrict__ err, int C, int k_max,
                                                     long long extra, int *__restrict__ npoints,
                                                     int *__restrict__ points_used, bool cached,
-                                                    unsigned long long *skeys)
+                                                    unsigned *skeys)
 {
-    __shared__ unsigned int hist[256];
-    __shared__ unsigned long long witness[256];
-    __shared__ unsigned long long s_prefix, s_T, s_total;
+    __shared__ unsigned hist[SEL_BUCKETS];
+    __shared__ unsigned long long list[SEL_LIST];
+    __shared__ unsigned long long w_total[32], s_T;
+    __shared__ unsigned w_min[32], w_max[32], w_sum[32];
     __shared__ long long s_rem;
-    __shared__ int s_done, s_used;
+    __shared__ unsigned s_bucket, s_count;
+    __shared__ int s_nlist, s_used;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int KM1 = k_max - 1;
     // the cached keys within the launch's shared memory, else read again from err
-    if (cached && !MPQ_CHECK_SMEM_END(8 * (size_t)C * KM1)) cached = false;
+    if (cached && !MPQ_CHECK_SMEM_END(4 * (size_t)C * KM1)) cached = false;
 
     if (tid == 0) {
-        s_total = 0;
         s_used = 0;
-        s_done = 0;
-        s_prefix = 0;
+        s_nlist = 0;
+    }
+    hist[tid] = 0u;
+    hist[tid + AB_THREADS] = 0u;
+    // the keys; how many there are, and their range
+    unsigned long long mine = 0;
+    unsigned kmin = NO_KEY, kmax = 0u;
+    for (int k = tid; k < C; k += AB_THREADS)
+        channel_keys(err, k, k_max, [&](int n, unsigned hi) {
+            if (cached) skeys[(size_t)k * KM1 + (n - 2)] = hi;
+            if (hi != NO_KEY) {
+                ++mine;
+                kmin = min(kmin, hi);
+                kmax = max(kmax, hi);
+            }
+        });
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+        w_total[warp] = mine;
+        w_min[warp] = kmin;
+        w_max[warp] = kmax;
     }
     __syncthreads();
-    unsigned long long mine = 0;
-    for (int k = tid; k < C; k += AB_THREADS)
-        channel_keys(err, k, k_max, [&](int n, unsigned long long key) {
-            if (cached) skeys[(size_t)k * KM1 + (n - 2)] = key;
-            mine += key != NO_KEY;
-        });
-    atomicAdd(&s_total, mine);
-    __syncthreads();
-    const long long total = (long long)s_total;
+    mine = w_total[lane];
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    kmin = __reduce_min_sync(0xffffffffu, w_min[lane]);
+    kmax = __reduce_max_sync(0xffffffffu, w_max[lane]);
+    const long long total = (long long)mine;
     const long long take = extra < total ? extra : total;
 
     // visit every selectable key
     auto for_keys = [&](auto f) {
         if (cached) {
-            const long long nk = (long long)C * KM1;
-            for (long long i = tid; i < nk; i += AB_THREADS) {
-                const unsigned long long key = skeys[i];
-                if (key != NO_KEY) f(key);
+            const int nk = C * KM1;
+            for (int i = tid; i < nk; i += AB_THREADS) {
+                const unsigned hi = skeys[i];
+                if (hi != NO_KEY) f(((unsigned long long)hi << 32) | (unsigned)i);
             }
         } else {
             for (int k = tid; k < C; k += AB_THREADS)
-                channel_keys(err, k, k_max, [&](int, unsigned long long key) {
-                    if (key != NO_KEY) f(key);
+                channel_keys(err, k, k_max, [&](int n, unsigned hi) {
+                    if (hi != NO_KEY)
+                        f(((unsigned long long)hi << 32) |
+                          (unsigned)((unsigned long long)k * KM1 + (n - 2)));
                 });
         }
     };
 
     unsigned long long T = 0;   // selected = keys <= T (when take > 0)
     if (take > 0 && take == total) {
-        T = NO_KEY - 1;
+        T = ~0ULL;
     } else if (take > 0) {
-        if (tid == 0) s_rem = take;   // 1-based rank of the key we look for
-        for (int shift = 56; shift >= 0; shift -= 8) {
-            for (int b = tid; b < 256; b += AB_THREADS) hist[b] = 0;
-            __syncthreads();
-            const unsigned long long prefix = s_prefix;
-            const int hs = shift + 8;
+        long long rem = take;   // 1-based rank of the wanted key among the `count` in [base, base + width]
+        unsigned long long count = (unsigned long long)total;
+        unsigned long long base = (unsigned long long)kmin << 32;
+        unsigned long long width = ((unsigned long long)(kmax - kmin) << 32) | 0xFFFFFFFFull;
+        while (count > SEL_LIST) {
+            // (hist is clear) buckets of 2^shift: at most SEL_BUCKETS of them
+            const int shift = max(0, 64 - __clzll((long long)width) - 11);
             for_keys([&](unsigned long long key) {
-                if (hs < 64 && ((key ^ prefix) >> hs) != 0) return;
-                const unsigned b = (unsigned)(key >> shift) & 255u;
-                atomicAdd(&hist[b], 1u);
-                witness[b] = key;   // meaningful only when the bucket ends with one key
+                if (key - base <= width) atomicAdd(&hist[(unsigned)((key - base) >> shift)], 1u);
             });
             __syncthreads();
-            if (warp == 0) {
-                // warp-parallel search for the bucket that holds the rem-th key
-                const long long rem = s_rem;
-                unsigned int loc = 0;
+            // the bucket that holds the rem-th key
+            const unsigned c0 = hist[2 * tid], c1 = hist[2 * tid + 1];
+            unsigned incl = c0 + c1;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) loc += hist[lane * 8 + i];
-                unsigned long long incl = loc;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                const unsigned long long excl = incl - loc;
-                const unsigned hit = __ballot_sync(0xffffffffu,
-                                                   (long long)excl < rem && rem <= (long long)incl);
-                const int src = __ffs(hit) - 1;
-                if (lane == src) {
-                    long long cum = (long long)excl;
-                    int b = lane * 8;
-                    for (; b < lane * 8 + 7; ++b) {
-                        if (cum + (long long)hist[b] >= rem) break;
-                        cum += hist[b];
-                    }
-                    s_rem = rem - cum;
-                    s_prefix = prefix | ((unsigned long long)b << shift);
-                    if (hist[b] == 1) {
-                        s_T = witness[b];
-                        s_done = 1;
-                    }
-                }
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
             }
+            if (lane == 31) w_sum[warp] = incl;
             __syncthreads();
-            if (s_done) break;
+            const unsigned long long before =
+                __reduce_add_sync(0xffffffffu, lane < warp ? w_sum[lane] : 0u) +
+                (unsigned long long)(incl - c0 - c1);
+            const long long want = rem - (long long)before;
+            if (want > 0 && want <= (long long)(c0 + c1)) {
+                const bool second = want > (long long)c0;
+                s_bucket = 2 * tid + (second ? 1 : 0);
+                s_count = second ? c1 : c0;
+                s_rem = want - (second ? (long long)c0 : 0);
+            }
+            hist[2 * tid] = 0u;
+            hist[2 * tid + 1] = 0u;
+            __syncthreads();
+            rem = s_rem;
+            count = s_count;
+            base += (unsigned long long)s_bucket << shift;
+            width = shift > 0 ? (1ULL << shift) - 1 : 0;
         }
-        T = s_done ? s_T : s_prefix;
+        // the keys left, and the one with rem - 1 smaller ones
+        for_keys([&](unsigned long long key) {
+            if (key - base <= width) {
+                const int at = atomicAdd(&s_nlist, 1);
+                if (MPQ_IN(at, SEL_LIST)) list[at] = key;
+            }
+        });
+        __syncthreads();
+        const int m = (int)count;
+        if (tid < m) {
+            const unsigned long long key = list[tid];
+            int smaller = 0;
+#pragma unroll 8
+            for (int i = 0; i < m; ++i) smaller += list[i] < key;
+            if (smaller == (int)(rem - 1)) s_T = key;
+        }
+        __syncthreads();
+        T = s_T;
     }
 
     // n_k = 1 + number of selected keys of channel k (a prefix n = 2..n_k, since p is monotone)
@@ -161,22 +191,22 @@ __device__ __forceinline__ void allocate_budget_cta(const float *__restrict__ er
     for (int k = tid; k < C; k += AB_THREADS) {
         int n_k = 1;
         if (take > 0) {
+            const unsigned long long first = (unsigned long long)k * KM1;
+            auto selected = [&](int n, unsigned hi) {
+                n_k += hi != NO_KEY &&
+                       (((unsigned long long)hi << 32) | (unsigned)(first + (n - 2))) <= T;
+            };
             if (cached) {
-                for (int n = 0; n < KM1; ++n) {
-                    const unsigned long long key = skeys[(size_t)k * KM1 + n];
-                    if (key != NO_KEY && key <= T) ++n_k;
-                }
+                for (int n = 2; n <= k_max; ++n) selected(n, skeys[first + (n - 2)]);
             } else {
-                channel_keys(err, k, k_max, [&](int, unsigned long long key) {
-                    if (key != NO_KEY && key <= T) ++n_k;
-                });
+                channel_keys(err, k, k_max, selected);
             }
         }
         npoints[k] = n_k;
         used += n_k;
     }
     if (points_used) {
-        for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(0xffffffffu, used, o);
+        used = __reduce_add_sync(0xffffffffu, used);
         if (lane == 0) atomicAdd(&s_used, used);   // integer sum: order-free
         __syncthreads();
         if (tid == 0) *points_used = s_used;
@@ -187,7 +217,7 @@ __global__ void __launch_bounds__(AB_THREADS)
 allocate_budget_kernel(const float *__restrict__ err, int C, int k_max, long long extra,
                        int *__restrict__ npoints, int *__restrict__ points_used, bool cached)
 {
-    extern __shared__ unsigned long long skeys[];   // [C * (k_max - 1)] when cached
+    extern __shared__ unsigned skeys[];   // [C * (k_max - 1)] when cached
     allocate_budget_cta(err, C, k_max, extra, npoints, points_used, cached, skeys);
 }
 
@@ -237,7 +267,7 @@ struct AllocBatch {
 __global__ void __launch_bounds__(AB_THREADS)
 allocate_batch_kernel(const __grid_constant__ AllocBatch b, int k_max, int mode)
 {
-    extern __shared__ unsigned long long skeys[];
+    extern __shared__ unsigned skeys[];
     if (!MPQ_IN(blockIdx.x, MPQ_MAX_BATCH) || !MPQ_IN(b.order[blockIdx.x], MPQ_MAX_BATCH)) return;
     const int l = b.order[blockIdx.x];
     if (mode == MPQ_ALLOC_BUDGET)
@@ -280,10 +310,11 @@ mpq_status launch_allocate_budget(const float *err, int C, int k_max, long long 
 {
     const long long nkeys = (long long)C * (k_max - 1);
     const bool cached = nkeys <= KEY_CACHE;
-    const size_t smem = cached ? (size_t)nkeys * sizeof(unsigned long long) : 0;
-    // always set: the kernel's static shared memory counts against the 48 KB default too
+    const size_t smem = cached ? (size_t)nkeys * sizeof(unsigned) : 0;
+    // always the same limit: calls of other threads may come between this and the launch
     cudaError_t e = cudaFuncSetAttribute(allocate_budget_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         KEY_CACHE * (int)sizeof(unsigned));
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
     allocate_budget_kernel<<<1, AB_THREADS, smem, stream>>>(err, C, k_max, extra, npoints,
                                                             points_used, cached);
@@ -308,8 +339,7 @@ mpq_status launch_allocate_batch(int n, const float *const *err, const int *C, i
         const long long nkeys = (long long)C[l] * (k_max - 1);
         const bool cached = mode == MPQ_ALLOC_BUDGET && nkeys <= KEY_CACHE;
         b.cached[l] = cached;
-        if (cached && (size_t)nkeys * sizeof(unsigned long long) > smem)
-            smem = (size_t)nkeys * sizeof(unsigned long long);
+        if (cached && (size_t)nkeys * sizeof(unsigned) > smem) smem = (size_t)nkeys * sizeof(unsigned);
         b.order[m++] = (unsigned char)l;
     }
     if (m == 0) return MPQ_OK;
@@ -322,7 +352,7 @@ mpq_status launch_allocate_batch(int n, const float *const *err, const int *C, i
         }
     const cudaError_t e = cudaFuncSetAttribute(allocate_batch_kernel,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+                                               KEY_CACHE * (int)sizeof(unsigned));
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
     allocate_batch_kernel<<<m, AB_THREADS, smem, stream>>>(b, k_max, mode);
     return cuda_status(cudaGetLastError(), "batched allocation kernel launch");
