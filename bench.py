@@ -34,6 +34,7 @@ UNIT = "elem*cand*pt/s"
 PROFILES = os.path.join(ROOT, "profiles")
 KERNEL_SOURCES = {
     "output_error": ("paper_2002_09049_gb300/csrc/output_error.cu",
+                     "paper_2002_09049_gb300/csrc/output_error_chain.cu",
                      "paper_2002_09049_gb300/csrc/output_error_f16.cu",
                      "paper_2002_09049_gb300/csrc/output_error_pair.cu",
                      "paper_2002_09049_gb300/csrc/pair_common.cuh",
@@ -477,10 +478,10 @@ def dominant_roofline(dominant, fam_ms, fam_work, peaks, peak_src, wl, args, sm_
     if dominant == "output_error":
         peak = peaks["bf16_tflops"]
         ach = fam_work[dominant] / t_s / 1e12
-        return {"kernel": "output_error_f16_kernel (Eq. 11, tcgen05 cta_group::2 kind::f16, "
-                          "scaled fp16 hi/lo operands, 3 passes, X split ahead; after "
-                          "pair_range_kernel and f16_split_kernel; output_error_tc_kernel for rows "
-                          "not 16-byte multiples)",
+        return {"kernel": "output_error_chain_kernel (Eq. 11, tcgen05 cta_group::2 kind::f16: the "
+                          "points' codes and the last residual's hi/lo halves against X's, 2 (k_max "
+                          "+ 2) row passes; after pair_range_kernel and f16_split_kernel; "
+                          "output_error_tc_kernel for rows not 16-byte multiples)",
                 "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "traffic": traffic,
                 "peak_source": f"{peak_src} bf16 dense burst (the fp16 rate of kind::f16)"}
@@ -914,7 +915,7 @@ def run_clip(args, world, rank, local):
     t1 = float(np.mean(one_ms)) / 1e3
     peak = peaks["bf16_tflops"]
     ach = flops_per_step / t1 / 1e12
-    roofline = {"kernel": "output_error_f16_kernel in clip mode (Eq. 12 residuals written once as "
+    roofline = {"kernel": "clip_error_kernel (Eq. 12 residuals written once as "
                           "fp16 hi/lo planes by clip_planes_kernel and tile-copied into a tcgen05 "
                           "cta_group::2 kind::f16 3-pass contraction) + candidate, X range, X split "
                           "and argmin kernels",

@@ -123,7 +123,8 @@ mpq_status mpq_quantize_layer(const float *W, int C, int d, int bits, int G,
  *
  * Scratch: with groups == 1, d a multiple of 16 and X, W, codes 16-byte aligned (the tensor-core
  * path with scaled fp16 operands), the call takes 4 (1 + C (k_max+1)) bytes (4 bytes with rmax),
- * rounded up to 256, plus 4 N d bytes for X's fp16 hi/lo planes
+ * rounded up to 256, plus 4 N d bytes for X's fp16 hi/lo planes, plus partial sums: 8 + 16384 bytes
+ * per tile of 2 floor(128 / (k_max + 2)) channels (8 bytes where N <= 256)
  * from the current device's default stream-ordered memory pool with cudaMallocAsync on `stream`
  * and returns them with cudaFreeAsync on `stream` -- concurrent calls on other streams each get
  * their own, and a CUDA graph capture records them as the graph's allocation nodes.
@@ -172,7 +173,7 @@ mpq_status mpq_quantize_layer_adaptive(const float *W, int C, int d, int bits, i
                                        float *scales, float *resid_sq, long long *ncand,
                                        void *stream);
 
-/* Words of mpq_output_error_noalloc's fixed scratch buffer (4 MiB). */
+/* Words of mpq_output_error_noalloc's fixed range table (4 MiB). */
 #define MPQ_NOALLOC_RANGE_WORDS (1 << 20)
 
 /*
@@ -182,10 +183,11 @@ mpq_status mpq_quantize_layer_adaptive(const float *W, int C, int d, int bits, i
  * framework whose allocator owns the stream-ordered pool, or a pool that is switched off.
  *
  * Same arguments (without rmax: the ranges are always measured), layouts, validation, results
- * (bit for bit) and errors as mpq_output_error, except for the scratch: the tensor-core path's range table (1 + C (k_max+1) words) lives in one
- * fixed device array of MPQ_NOALLOC_RANGE_WORDS words (4 MiB) inside the library, which every
- * device that loads the library's module keeps until the process exits.  The call zeroes the
- * part of the table it uses before filling it.  Therefore:
+ * (bit for bit) and errors as mpq_output_error, except for the scratch: the tensor-core path's
+ * range table (1 + C (k_max+1) words, MPQ_NOALLOC_RANGE_WORDS at most: 4 MiB) and its partial sums
+ * (4 MiB) live in one fixed device array inside the library, which every device that loads the
+ * library's module keeps until the process exits.  The call zeroes the part of the table it uses
+ * before filling it.  Therefore:
  *  - a call whose table would exceed MPQ_NOALLOC_RANGE_WORDS words is rejected with
  *    MPQ_ERR_UNSUPPORTED before anything is enqueued;
  *  - the first call on a device (made with that device current) looks up the array's device

@@ -192,7 +192,8 @@ extern "C" mpq_status mpq_output_error(const float *X, int N, int groups, const 
 // (overlapping calls race on it, as its declaration states).  Host code cannot use the symbol
 // itself as a device address: its address on each device is resolved once, with that device
 // current, by the first call made there, and kept.
-static __device__ __align__(256) unsigned g_noalloc_range[MPQ_NOALLOC_RANGE_WORDS];
+static __device__ __align__(256) unsigned g_noalloc_range[MPQ_NOALLOC_RANGE_WORDS +
+                                                          CHAIN_FIXED_SCRATCH / 4];
 static unsigned *g_noalloc_addr[kMaxDevices];
 static std::mutex g_noalloc_mu;
 

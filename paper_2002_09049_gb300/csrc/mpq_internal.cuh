@@ -61,6 +61,10 @@ mpq_status launch_output_error(const float *X, int N, int groups, const float *W
                                const int8_t *codes, const float *scales, int C, int d, int k_max,
                                float *err, cudaStream_t stream, unsigned *range = nullptr,
                                const float *rmax = nullptr);
+// Scratch of the contraction's partial sums (output_error_chain.cu) that callers of
+// launch_output_error with a range table of their own hold after its MPQ_NOALLOC_RANGE_WORDS words
+// (larger layers leave each channel tile to one CTA pair).
+constexpr size_t CHAIN_FIXED_SCRATCH = 1 << 22;
 // Words of range scratch a call needs (0 where it takes no scratch).
 size_t output_error_scratch_words(const float *X, int groups, const float *W,
                                   const int8_t *codes, int C, int d, int k_max);

@@ -1,6 +1,6 @@
-// Pieces shared by the CTA-pair output-error kernels (Sec. 3.3, Eq. 11): the power-of-two scaling
-// and fp16 hi/lo split of the contraction's operands, the pairing of a warp's two channels for
-// conflict-free operand stores, and tile-map encoding for the TMA copies.
+// Pieces shared by the CTA-pair output-error kernels (Sec. 3.3, Eq. 11 and 12): the power-of-two
+// scaling and fp16 hi/lo split of the contraction's operands, and tile-map encoding for the TMA
+// copies.
 #pragma once
 
 #include <cuda.h>
@@ -42,25 +42,6 @@ __device__ __forceinline__ void split_f16x2(float a, float b, uint32_t &hi, uint
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
-// fp16 operand stores fill 64-byte half rows of a 128-byte-swizzled tile, and the swizzle puts a
-// half row in banks 0-15 or 16-31 by bit 2 of its row.  The two channels of a warp's residual
-// items (slots j = 2t, 2t+1: lanes 0-15 and 16-31) are D apart, with D (k_max+1) = 4 (mod 8) where
-// possible, so that their rows differ in bit 2.  A bijection of the slots 0..nch-1: blocks of 2D
-// slots pair channel i with i + D; a last partial block of T slots pairs its first T - D channels
-// so and keeps the rest in place.
-template <int KP1>
-__device__ __forceinline__ int pair_channel(int j, int nch)
-{
-    constexpr int D = (KP1 & 1) ? 4 : ((KP1 & 3) == 2 ? 2 : 1);
-    const int F = nch / (2 * D) * (2 * D);
-    if (j < F) {
-        const int w = j % (2 * D);
-        return j - w + (w >> 1) + (w & 1) * D;
-    }
-    const int T = nch - F, m = T > D ? T - D : 0, s = j - F;
-    return s < 2 * m ? F + (s >> 1) + (s & 1) * D : F + m + (s - 2 * m);
-}
-
 // Host: tile map over a row-major tensor (dims[0] contiguous, byte strides for dims 1..), zero
 // fill out of range, the given shared-memory swizzle.  False if the driver entry point is missing
 // or rejects the arguments.
@@ -71,12 +52,23 @@ bool encode_tile_map(CUtensorMap *m, CUtensorMapDataType type, int rank, const v
 // Host: max|X| (float bits) into range[0], zeroed first (N d a multiple of 4, X 16-byte aligned).
 mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, cudaStream_t stream);
 
-// Host: the output error of the greedy residuals on output_error_f16.cu's kernel, with its range
-// table ready on `stream` (xrange[0] = max|X|, vrange = max|r| per residual vector, float bits)
-// and `xs` scratch of 2 N d fp16 for the split X planes.
-mpq_status launch_output_error_f16(const float *X, int N, const float *W, const int8_t *codes,
-                                   const float *scales, int C, int d, int k_max, float *err,
-                                   const unsigned *xrange, const unsigned *vrange, uint16_t *xs,
-                                   cudaStream_t stream);
+// Host: X * 2^e (e from xrange[0]) split into the fp16 hi and lo planes xs ([2][N][d]).
+cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange, uint16_t *xs,
+                           cudaStream_t stream);
+
+// Host: the output error of the greedy points (output_error_chain.cu), with its ranges ready on
+// `stream` (xrange[0] = max|X|, vrange = max|r| per residual vector, float bits); xs: the split X
+// planes, or NULL (the contraction then splits X itself); part: part_bytes of 256-byte aligned
+// scratch for partial sums, at least chain_count_bytes(tiles) and that much of it zeroed on
+// `stream` (chain_scratch_bytes(tiles, chain_max_gang(N)) is all it can use).
+mpq_status launch_output_error_chain(const float *X, int N, const float *W, const int8_t *codes,
+                                     const float *scales, int C, int d, int k_max, float *err,
+                                     const unsigned *xrange, const unsigned *vrange,
+                                     const uint16_t *xs, void *part, size_t part_bytes,
+                                     cudaStream_t stream);
+int chain_tiles(int C, int k_max);   // channel tiles of a CTA pair
+size_t chain_count_bytes(int tiles);
+size_t chain_scratch_bytes(int tiles, int gang);
+int chain_max_gang(int N);
 
 }  // namespace mpq

@@ -136,3 +136,43 @@ def test_ranges_from_the_greedy_search(gpu, oracle, C, d, N, K, bits):
     keep = np.arange(C) != 1
     e_or = oracle.output_error(X, 1, W[keep], o["codes"][:, keep], o["scales"][keep], K)
     compare_err(e1.cpu().numpy()[keep], e_or)
+
+
+# channel tiles are 2 floor(128 / (k_max + 2)) channels (24 at k_max = 8), row tiles 256 calibration
+# rows, steps 64 elements: one less, exactly and one more of each; every row tile in one CTA pair
+# or shared by several; the largest k_max
+@pytest.mark.parametrize("C,d,N,K", [(24, 64, 256, 8), (23, 48, 255, 8), (25, 80, 257, 8),
+                                     (84, 16, 70, 1), (85, 272, 513, 1), (7, 320, 2049, 16),
+                                     (33, 1040, 1500, 6), (2000, 64, 700, 4)])
+def test_point_chain_tiles(gpu, oracle, C, d, N, K):
+    """The contraction over the points (codes and the last residual): tile edges, through the
+    pooled and the fixed-scratch entry point (bit for bit the same), against the oracle."""
+    W = wlm.random_weights(C, d, C + d + K, "t")
+    X = wlm.random_calibration(N, d, 9 + d)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(gpu)
+    codes, scales, _, _ = binding.mpq_quantize_layer(t(W), 4, 32, K)
+    e = binding.mpq_output_error(t(X), t(W), codes, scales, K)
+    e_fixed = binding.mpq_output_error_noalloc(t(X), t(W), codes, scales, K)
+    torch.cuda.synchronize()
+    assert torch.equal(e, e_fixed)
+    some = np.unique(np.concatenate([np.arange(min(C, 30)), np.arange(max(0, C - 30), C)]))
+    q, s = codes.cpu().numpy()[:, some], scales.cpu().numpy()[some]
+    compare_err(e.cpu().numpy()[some], oracle.output_error(X, 1, W[some], q, s, K))
+
+
+@pytest.mark.parametrize("K", [1, 5, 16])
+def test_codes_that_are_not_nearest_values(gpu, oracle, K):
+    """Codes and scales of the caller's own, under which residuals grow: those channels take plain
+    fp32 sums, the others (nearest codes) the chain."""
+    C, d, N = 60, 144, 300
+    rng = np.random.default_rng(K)
+    W = wlm.random_weights(C, d, 21, "normal")
+    q = oracle.quantize_layer(W, 4, 32, K)
+    codes, scales = q["codes"].copy(), q["scales"].copy()
+    for k in (0, 3, 41, 59):
+        codes[:, k] = rng.integers(-7, 8, size=(K, d)).astype(np.int8)
+        scales[k] = (10.0 ** rng.uniform(0, 3, size=K)).astype(np.float32)
+    codes[:, 7] = 0
+    scales[7] = 1e30                                   # a scale far above its residual, codes 0
+    X = wlm.random_calibration(N, d, 5)
+    compare_err(gpu_err(X, W, codes, scales, K), oracle.output_error(X, 1, W, codes, scales, K))
