@@ -123,3 +123,24 @@ def test_adaptive_tiny_gap_zero_scales(gpu, oracle):
         assert np.any(np.float32(o["gamma"][:, 0] / (2 ** (bits - 1) - 1)) == 0.0)
         g = run(W, bits, 3, max_cand=10 ** 7)
         compare_adaptive(g, o, bits, oracle)
+
+
+@pytest.mark.parametrize("C,d,bits,k_max,kind", [
+    (4, 73, 4, 2, "normal"),      # 511 thresholds: all of them listed
+    (4, 74, 4, 2, "normal"),      # 518: counted in buckets first
+    (3, 640, 4, 2, "lattice"),    # equal magnitudes by the hundred: the sort list overflows
+    (3, 700, 3, 2, "binades"),    # magnitudes over 24 binades, ties in the norm's additions
+    (2, 130, 7, 2, "tails"),      # Qmax = 63 and outliers: scales far below the largest weight
+])
+def test_adaptive_bucket_screen(gpu, oracle, C, d, bits, k_max, kind):
+    """The bucket screen's edges: row lengths on both sides of its rule, rows whose candidate
+    thresholds do not fit the sort list, wide ranges of magnitudes."""
+    rng = np.random.default_rng(d)
+    W = rng.standard_normal((C, d)).astype(np.float32)
+    if kind == "lattice":
+        W = (np.round(W * 4) / 4).astype(np.float32)
+    elif kind == "binades":
+        W = (np.float32(1.5) * np.exp2(rng.integers(-12, 12, (C, d)))).astype(np.float32)
+    elif kind == "tails":
+        W = np.where(rng.random((C, d)) < 0.02, W * 300, W).astype(np.float32)
+    check(oracle, W, bits, k_max, cap=BIG, piecewise=True)
