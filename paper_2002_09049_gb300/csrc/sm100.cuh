@@ -206,19 +206,7 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint6
         : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 with bf16 A and B (fp32 accumulate), one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                         uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// CTA-pair MMA of kind::f16 with fp16 A and B (fp32 accumulate), issued by one thread of the
+// CTA-pair MMA of kind::f16 (fp16 or bf16 A and B, as idesc says; fp32 accumulate), issued by one thread of the
 // pair's even CTA: A is M = 256 rows, 128 in each CTA's shared memory at the descriptor's offset;
 // B is N rows, N/2 in each CTA; D lands in each CTA's tensor memory (its own 128 rows x N columns)
 // at d_tmem.
@@ -312,25 +300,6 @@ __device__ __forceinline__ void tmem_st_32x32b_x4(uint32_t taddr, const float (&
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr),
                  "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
                  : "memory");
-}
-
-// Two loads of 32 columns (e.g. a segment and its running sums) in flight together, one wait.
-__device__ __forceinline__ void tmem_ld2_32x32b_x32(uint32_t taddr_a, uint32_t taddr_b,
-                                                    float (&a)[32], float (&b)[32])
-{
-    uint32_t x[32], y[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%64];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%65];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]), "=r"(x[14]), "=r"(x[15]), "=r"(x[16]), "=r"(x[17]), "=r"(x[18]), "=r"(x[19]), "=r"(x[20]), "=r"(x[21]), "=r"(x[22]), "=r"(x[23]), "=r"(x[24]), "=r"(x[25]), "=r"(x[26]), "=r"(x[27]), "=r"(x[28]), "=r"(x[29]), "=r"(x[30]), "=r"(x[31]), "=r"(y[0]), "=r"(y[1]), "=r"(y[2]), "=r"(y[3]), "=r"(y[4]), "=r"(y[5]), "=r"(y[6]), "=r"(y[7]), "=r"(y[8]), "=r"(y[9]), "=r"(y[10]), "=r"(y[11]), "=r"(y[12]), "=r"(y[13]), "=r"(y[14]), "=r"(y[15]), "=r"(y[16]), "=r"(y[17]), "=r"(y[18]), "=r"(y[19]), "=r"(y[20]), "=r"(y[21]), "=r"(y[22]), "=r"(y[23]), "=r"(y[24]), "=r"(y[25]), "=r"(y[26]), "=r"(y[27]), "=r"(y[28]), "=r"(y[29]), "=r"(y[30]), "=r"(y[31])
-        : "r"(taddr_a), "r"(taddr_b)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        a[i] = __uint_as_float(x[i]);
-        b[i] = __uint_as_float(y[i]);
-    }
 }
 
 // Stores 32 consecutive 32-bit columns of lanes (base .. base+31), one lane per thread.
@@ -507,6 +476,20 @@ __device__ __forceinline__ double ld_dsmem_f64(const double *local, uint32_t ran
     double v;
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote) : "memory");
     return v;
+}
+
+__device__ __forceinline__ void st_dsmem_u32(void *local, uint32_t rank, uint32_t v)
+{
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)),
+                 "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
+
+// This thread's writes before it ordered before its later ones, at cluster scope.
+__device__ __forceinline__ void fence_cluster()
+{
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
 }
 
 __device__ __forceinline__ void st_dsmem_f64(double *local, uint32_t rank, double v)

@@ -99,3 +99,55 @@ def test_full_size_sampled(gpu, oracle):
     for c0 in (0, 5000, 11008 - 16):
         ref = oracle.multipoint_linear(X, c_np, s_np, n_host, 16, channels=(c0, c0 + 16), threads=8)
         assert np.array_equal(Y[c0:c0 + 16], ref[c0:c0 + 16])
+
+
+@pytest.mark.parametrize("T", [1, 7, 8, 9, 16, 17, 33, 100])
+@pytest.mark.parametrize("d,bits,off", [(144, 4, 0), (152, 4, 0), (147, 4, 0), (145, 3, 1),
+                                        (8192, 8, 0), (8191, 8, 3)])
+def test_few_inputs_and_odd_rows(gpu, oracle, d, bits, off, T):
+    """The kernel for a few inputs and for rows and layers the tensor-memory kernel cannot take:
+    block edges of its inputs, row lengths and input addresses of every alignment (off: bytes into
+    a larger buffer), sums beyond 2^24 (a warp's fp32 share of a row stays below it), with and
+    without centres, R up to 16."""
+    k_max, C, p = 9, 37, 10
+    rng = np.random.default_rng(d + T)
+    q = 2 ** (bits - 1) - 1
+    codes = rng.choice(np.array([-q, q, 0, 1], np.int8), (k_max, C, d), p=[.45, .45, .05, .05])
+    scales = rng.uniform(0.0, 0.02, (C, k_max)).astype(np.float32)
+    center = rng.uniform(-0.1, 0.1, C).astype(np.float32)
+    npts = points(C, k_max, T, [0, 1, 2, 3, 5, 9])
+    X = rng.choice(np.array([-128, 127, 5], np.int8), (T, d))
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    buf = torch.zeros(T * d + off, dtype=torch.int8, device=DEV)
+    Xd = buf[off:].view(T, d)
+    Xd.copy_(t(X))
+    for cen in (None, center):
+        lay = binding.mpq_pack_layout(npts, d, k_max, bits, p, centered=cen is not None)
+        packed = binding.mpq_pack_points(t(codes), t(scales), npts, lay,
+                                         center=None if cen is None else t(cen))
+        Y = binding.mpq_multipoint_linear(Xd, lay, packed).cpu().numpy()
+        ref = oracle.multipoint_linear(X, codes, scales, npts, p, center=cen, threads=8)
+        assert np.array_equal(Y, ref)
+
+
+@pytest.mark.parametrize("C,d,T", [(3100, 64, 1024), (40, 1088, 3000), (2100, 320, 514),
+                                   (1500, 448, 777)])
+def test_pairs_and_rounds(gpu, oracle, C, d, T):
+    """The tensor-memory kernel: an odd number of row tiles, a second round of units, inputs not a
+    multiple of 4 (no 16-byte stores) or of 256, one chunk a unit, with centres."""
+    k_max, bits, p = 2, 4, 12
+    rng = np.random.default_rng(C)
+    codes = rng.integers(-7, 8, (k_max, C, d)).astype(np.int8)
+    scales = rng.uniform(0.0, 0.02, (C, k_max)).astype(np.float32)
+    center = rng.uniform(-0.1, 0.1, C).astype(np.float32)
+    npts = points(C, k_max, T)
+    X = rng.integers(-128, 128, (T, d)).astype(np.int8)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    lay = binding.mpq_pack_layout(npts, d, k_max, bits, p, centered=True)
+    packed = binding.mpq_pack_points(t(codes), t(scales), npts, lay, center=t(center))
+    Y = binding.mpq_multipoint_linear(t(X), lay, packed).cpu().numpy()
+    some = np.unique(np.concatenate([np.arange(24), rng.integers(0, C, 24), np.arange(C - 24, C)]))
+    some = some[(some >= 0) & (some < C)]
+    ref = oracle.multipoint_linear(X, np.ascontiguousarray(codes[:, some]), scales[some], npts[some],
+                                   p, center=center[some], threads=8)
+    assert np.array_equal(Y[some], ref)
