@@ -11,12 +11,10 @@
 //   E(s) = ||r - s q||^2 = ||r||^2 - 2 s P + s^2 N,   P = sum_j |r_j| c_j,   N = sum_j c_j^2,
 // so only D(s) = s (s N - 2 P) decides the argmin.  N is an exact integer and P is accumulated
 // exactly in 64-bit fixed point (|r_j| scaled by 2^S, S chosen per step from max|r| so the sum
-// cannot overflow; exact for every element whose code can be nonzero on the grid).  Every D is
-// first evaluated in fp32 together with a rigorous bound on its rounding error; only the
-// candidates whose interval can hold the minimum are re-evaluated in double, and the lowest index
-// among the exact minima wins.  The result is the argmin of the exact D values: deterministic and
-// independent of d and of the summation order, with the narrow fp64 pipe touched a few times per
-// step.
+// cannot overflow; exact for every element whose code can be nonzero on the grid).  Every
+// candidate's D is evaluated in double from them, and the lowest index among the exact minima wins.
+// The result is the argmin of the exact D values: deterministic and independent of d and of the
+// summation order.
 //
 // Event form.  The candidate scales increase with g, so every element's code c_j(g) is a
 // non-increasing step function of g (the fp32 quotient, rint and the clamp are all monotone).
@@ -74,6 +72,8 @@ constexpr int QNEAR = 128;   // lattice-adjacent elements a group queues per ste
 struct Scratch {
     float nearq[QNEAR];
     int nq;
+    unsigned pb[2];   // levels of queued elements held at the largest scale: P (two words), N
+    int nbase;
     float f[8];
     float v[8];
     unsigned long long key[8];
@@ -90,12 +90,14 @@ struct Scratch {
 // channel group (all 4-byte words): `copies` copies of hLo[G+1], hHi[G+1] (64-bit P bins as two
 // words) and hN[G+1], then r[d].  Without the lattice every warp has a private copy (so warps
 // never contend on a bin); with the lattice form (below) events are rare and the group shares one
-// copy, and the group also holds nb lattice buckets first, two words each: the low 32 bits of the
+// copy (every region a multiple of 16 bytes, cleared with 16-byte stores), and the group also holds nb lattice buckets first, two words each: the low 32 bits of the
 // bucket's fixed-point R sum, and its high bits plus the bucket's element count shifted to bit
 // cnt_bit (the launcher checks that neither field can overflow).  (Two separate word arrays, low
-// words on all 32 banks, measured no faster.)  Group regions stay 8-byte
-// aligned.
-__host__ __device__ constexpr size_t lattice_words(int nb) { return (size_t)2 * nb; }
+// words on all 32 banks, measured no faster.)
+__host__ __device__ constexpr size_t words4(size_t n) { return (n + 3) & ~(size_t)3; }
+__host__ __device__ constexpr size_t lattice_words(int nb) { return words4((size_t)2 * nb); }
+__host__ __device__ constexpr size_t table_bytes(int G) { return words4((size_t)2 * G) * 4; }
+__host__ __device__ constexpr size_t bin_words(int G, int copies) { return words4((size_t)3 * (G + 1) * copies); }
 
 // bytes of the CTA's bucket -> position-index table (uint16 per bucket, and 16 spare entries so
 // that the largest element's bucket, at most nb - 1, needs no clamp), 16-byte multiple
@@ -103,7 +105,7 @@ __host__ __device__ constexpr size_t lut_bytes(int nb) { return ((size_t)(nb + 1
 
 __host__ __device__ constexpr size_t group_words(int G, int d, int copies, int nb)
 {
-    return lattice_words(nb) + (((size_t)3 * (G + 1) * copies + (size_t)d + 1) & ~(size_t)1);
+    return lattice_words(nb) + bin_words(G, copies) + words4((size_t)d);
 }
 
 template <int WPC>
@@ -118,11 +120,9 @@ __device__ __forceinline__ void gsync(int grp)
     }
 }
 
-__device__ __forceinline__ float warp_max(float v)
+__device__ __forceinline__ float warp_max(float v)   // v >= 0 (its bits order like an integer's)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
 template <typename T>
@@ -130,13 +130,6 @@ __device__ __forceinline__ T warp_sum(T v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ float warp_min(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
@@ -191,21 +184,6 @@ __device__ __forceinline__ void group_sum2(long long &x, long long &y, Scratch &
     }
 }
 
-template <int WPC>
-__device__ __forceinline__ float group_min(float v, Scratch &sc, int gw, int lane, int grp)
-{
-    v = warp_min(v);
-    if (WPC > 1) {
-        gsync<WPC>(grp);
-        if (lane == 0) sc.f[gw] = v;
-        gsync<WPC>(grp);
-        v = sc.f[0];
-#pragma unroll
-        for (int i = 1; i < WPC; ++i) v = fminf(v, sc.f[i]);
-    }
-    return v;
-}
-
 // Order-preserving map of a double to unsigned 64-bit (total order, -0 < +0 is harmless here).
 __device__ __forceinline__ unsigned long long ordered_bits(double x)
 {
@@ -213,41 +191,37 @@ __device__ __forceinline__ unsigned long long ordered_bits(double x)
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
-__device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b)
-{
-    return a < b ? a : b;
-}
-
 // Group-wide lexicographic min of (D, g): smallest D, lowest g among equal D.  The double is
-// reduced as its order-preserving integer image (no fp64 compares), then the lowest g among the
-// lanes that hold that minimum.
+// reduced as its order-preserving integer image (no fp64 compares), word by word, and the warps'
+// minima in one exchange.
 template <int WPC>
 __device__ __forceinline__ int group_argmin(double D, int g, Scratch &sc, int gw, int lane,
                                             int grp)
 {
-    unsigned long long key = ordered_bits(D);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) key = umin64(key, __shfl_xor_sync(0xffffffffu, key, o));
+    const unsigned long long key = ordered_bits(D);
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
+    int mg = (int)__reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? (unsigned)g : ~0u);
     if (WPC > 1) {
         gsync<WPC>(grp);
-        if (lane == 0) sc.key[gw] = key;
+        if (lane == 0) {
+            sc.key[gw] = ((unsigned long long)mh << 32) | ml;
+            sc.g[gw] = mg;
+        }
         gsync<WPC>(grp);
-        key = sc.key[0];
+        unsigned long long best = sc.key[0];
+        mg = sc.g[0];
 #pragma unroll
-        for (int i = 1; i < WPC; ++i) key = umin64(key, sc.key[i]);
+        for (int i = 1; i < WPC; ++i) {
+            const unsigned long long k = sc.key[i];
+            if (k < best || (k == best && sc.g[i] < mg)) {
+                best = k;
+                mg = sc.g[i];
+            }
+        }
     }
-    int cand = (ordered_bits(D) == key) ? g : INT_MAX;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cand = min(cand, __shfl_xor_sync(0xffffffffu, cand, o));
-    if (WPC > 1) {
-        gsync<WPC>(grp);
-        if (lane == 0) sc.g[gw] = cand;
-        gsync<WPC>(grp);
-        cand = sc.g[0];
-#pragma unroll
-        for (int i = 1; i < WPC; ++i) cand = min(cand, sc.g[i]);
-    }
-    return cand;
+    return mg;
 }
 
 // In-place suffix sums over items t in [t0, t1) by the whole group: item t <- sum of items
@@ -440,14 +414,6 @@ __device__ __forceinline__ long long bin64(const unsigned int *hLo, const unsign
     return (long long)(((unsigned long long)hHi[t] << 32) | hLo[t]);
 }
 
-// Int64 -> fp32 without the fp64 pipe: two exact 32-bit halves, three roundings in total.
-__device__ __forceinline__ float i64_to_f32(long long x)
-{
-    const float hi = (float)(int)(x >> 32);
-    const float lo = (float)(unsigned int)x;
-    return __fmaf_rn(hi, 4294967296.0f, lo);
-}
-
 // Columns of tensor memory a CTA allocates for its groups' residual rows in the TM build: a power of
 // two, at least 32.
 __host__ __device__ constexpr uint32_t tm_alloc_cols(int cols)
@@ -499,7 +465,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
             ftab[G + g] = __frcp_rn(f);
         }
     // the last group's region ends the carve-up of dynamic shared memory
-    if (!MPQ_CHECK_SMEM_END((TABLE ? 8 * (size_t)G : 0) + (LAT ? lut_bytes(nb) : 0) +
+    if (!MPQ_CHECK_SMEM_END((TABLE ? table_bytes(G) : 0) + (LAT ? lut_bytes(nb) : 0) +
                             4 * (size_t)GPC * group_words(G, dsm, COPIES, nc)))
         return;
     auto fg = [&](int g) -> float { return TABLE ? ftab[g] : grid.frac(g, G); };
@@ -507,25 +473,35 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
     // Lattice compression: only the positions (g+1)(2L-1) are read, so bucket b is stored at the
     // index of the largest position <= b (lut[b]; nc positions in all): the suffix sum at a
     // position's index is the sum over the buckets at or above it, as before.
-    unsigned short *lut = reinterpret_cast<unsigned short *>(ftab + (TABLE ? 2 * G : 0));
+    unsigned short *lut = reinterpret_cast<unsigned short *>(ftab + (TABLE ? table_bytes(G) / 4 : 0));
     if (LAT) {
-        for (int b = threadIdx.x; b < nb; b += QTHREADS) lut[b] = 0;
+        __shared__ int s_sum[QTHREADS / 32];
+        for (int b = threadIdx.x; b < (int)(lut_bytes(nb) / 4); b += QTHREADS)
+            reinterpret_cast<unsigned *>(lut)[b] = 0u;
         __syncthreads();
         for (int x = threadIdx.x; x < G * qmax; x += QTHREADS) {
             const int g = x / qmax, L = x - g * qmax + 1;
             if (MPQ_IN((g + 1) * (2 * L - 1), nb)) lut[(g + 1) * (2 * L - 1)] = 1;
         }
         __syncthreads();
-        if (warp == 0) {   // inclusive count of positions, minus one
-            int run = 0;
-            for (int b0 = 0; b0 < nb; b0 += 32) {
-                const int b = b0 + lane;
-                const int bit = b < nb ? lut[b] : 0;
-                const unsigned bal = __ballot_sync(0xffffffffu, bit);
-                const int incl = run + __popc(bal & ((2u << lane) - 1u));
-                if (b < nb) lut[b] = (unsigned short)(incl - 1);
-                run += __popc(bal);
-            }
+        // inclusive count of positions, minus one: a contiguous block of buckets per thread
+        const int per = (nb + QTHREADS - 1) / QTHREADS;
+        const int b0 = min(nb, (int)threadIdx.x * per), b1 = min(nb, b0 + per);
+        int own = 0;
+        for (int b = b0; b < b1; ++b) own += lut[b];
+        int run = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += y;
+        }
+        if (lane == 31) s_sum[warp] = run;
+        __syncthreads();
+        run -= own + 1;
+        for (int w = 0; w < warp; ++w) run += s_sum[w];
+        for (int b = b0; b < b1; ++b) {
+            run += lut[b];
+            lut[b] = (unsigned short)run;
         }
     }
     // TM: the CTA's tensor memory for its groups' rows (warp 0 allocates and releases it)
@@ -553,7 +529,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
     unsigned int *mLo = gbase;
     unsigned int *mHi = mLo + (G + 1);
     int *mN = reinterpret_cast<int *>(mHi + (G + 1));
-    float *sr = reinterpret_cast<float *>(gbase + (size_t)3 * (G + 1) * COPIES);
+    float *sr = reinterpret_cast<float *>(gbase + bin_words(G, COPIES));
     Scratch &sc = scratch[grp];
 
     const size_t plane = (size_t)C * d;
@@ -646,21 +622,27 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
             // (|r| >= smax / 2G) and below 2^lat_bits; elsewhere sum_j R_j c_j < 2^62
             const bool zs = __fmul_rn(fg(0), smax) == 0.0f;
             const int S = (LAT && !zs) ? lat_bits - e : 62 - e - hbits;
-            const float pscale = ldexpf(1.0f, -S - e);   // P 2^-S / 2^e for the fp32 screen
             // lattice elements (|r| >= smax / 2G >= 2^(e - 2 - log2(2 G Qmax))) are normal floats
             // unless max|r| itself is below ~2^-100
             const bool lat_normal = LAT && !zs && e > -100;
             const double down = pow2d(-S);
-            const float smax_e = ldexpf(smax, -e);   // smax / 2^e for the fp32 screen
             if (!direct) {
-                for (int t = COPIES > 1 ? lane : gt; t <= G; t += COPIES > 1 ? 32 : NT) {
-                    hLo[t] = 0u;   // each warp clears its own copy, or the group the shared one
-                    hHi[t] = 0u;
-                    hN[t] = 0;
+                if (COPIES > 1) {
+                    for (int t = lane; t <= G; t += 32) {   // each warp clears its own copy
+                        hLo[t] = 0u;
+                        hHi[t] = 0u;
+                        hN[t] = 0;
+                    }
+                } else {   // lattice (none without it) and bins are adjacent
+                    uint4 *z = reinterpret_cast<uint4 *>(gl);
+                    const int n4 = (int)((lattice_words(nc) + bin_words(G, 1)) / 4);
+                    for (int t = gt; t < n4; t += NT) z[t] = make_uint4(0u, 0u, 0u, 0u);
                 }
-                if (LAT) {
-                    for (int t = gt; t < 2 * nc; t += NT) lat[t] = 0u;
-                    if (gt == 0) sc.nq = 0;
+                if (LAT && gt == 0) {
+                    sc.nq = 0;
+                    sc.pb[0] = 0u;
+                    sc.pb[1] = 0u;
+                    sc.nbase = 0;
                 }
                 gsync<WPC>(grp);
             }
@@ -853,7 +835,20 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                         if (a != 0.0f) events(a);
                     }
                 }
-                group_sum2<WPC>(Pb, Nb, sc, gw, lane, grp);   // publishes the bins too
+                if (LAT) {   // only queued elements contribute here: few, if any
+                    if (Pb != 0 || Nb != 0) {
+                        add64(&sc.pb[0], &sc.pb[1], (unsigned int)Pb,
+                              (unsigned int)((unsigned long long)Pb >> 32));
+                        atomicAdd(&sc.nbase, (int)Nb);
+                    }
+                    gsync<WPC>(grp);   // publishes the bins too
+                    if (!direct) {
+                        Pb = (long long)(((unsigned long long)sc.pb[1] << 32) | sc.pb[0]);
+                        Nb = sc.nbase;
+                    }
+                } else {
+                    group_sum2<WPC>(Pb, Nb, sc, gw, lane, grp);   // publishes the bins too
+                }
                 const long long Pbase = Pb, Nbase = Nb;
                 // ---- suffix sums over the event bins (private copies, if any, merged into
                 // copy 0; warp 0), in place: bin t <- sum of bins u >= t, so P_g = Pbase +
@@ -877,13 +872,13 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                     mN[t] = (int)q;
                 };
                 auto lat_load = [&](int t, unsigned long long &p, long long &q) {
-                    const unsigned hi = lat[2 * t + 1];
-                    p = ((unsigned long long)(hi & hmask) << 32) | lat[2 * t];
-                    q = hi >> cnt_bit;
+                    const uint2 v = reinterpret_cast<const uint2 *>(lat)[t];
+                    p = ((unsigned long long)(v.y & hmask) << 32) | v.x;
+                    q = v.y >> cnt_bit;
                 };
                 auto lat_store = [&](int t, unsigned long long p, long long q) {
-                    lat[2 * t] = (unsigned)p;
-                    lat[2 * t + 1] = (unsigned)(p >> 32) | ((unsigned)q << cnt_bit);
+                    reinterpret_cast<uint2 *>(lat)[t] =
+                        make_uint2((unsigned)p, (unsigned)(p >> 32) | ((unsigned)q << cnt_bit));
                 };
                 // with the lattice: warp 0 scans the bins while the other warps scan the lattice
                 // together (named barrier 8 + grp: gsync takes 0 or 1..4), or one warp both;
@@ -912,9 +907,9 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                         for (int L = 1; L <= qmax; ++L) {
                             const int b = lut[(g + 1) * (2 * L - 1)];
                             if (!MPQ_IN(b, nc)) continue;
-                            const unsigned hi = lat[2 * b + 1];
-                            p += (long long)(((unsigned long long)(hi & hmask) << 32) | lat[2 * b]);
-                            n += (long long)(2 * L - 1) * (hi >> cnt_bit);
+                            const uint2 v = reinterpret_cast<const uint2 *>(lat)[b];
+                            p += (long long)(((unsigned long long)(v.y & hmask) << 32) | v.x);
+                            n += (long long)(2 * L - 1) * (v.y >> cnt_bit);
                         }
                         mLo[g + 1] = (unsigned int)p;
                         mHi[g + 1] = (unsigned int)((unsigned long long)p >> 32);
@@ -922,34 +917,14 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                     }
                     gsync<WPC>(grp);
                 }
-                // ---- fp32 screen of D / 2^2e = s'(s'N - 2P') with s' = s / 2^e and
-                // P' = P 2^-S / 2^e (both O(1) by construction): keep every candidate whose error
-                // interval can contain the minimum, then decide among those in double.  The
-                // inputs carry at most ~8 roundings of 2^-24, the bound allows 2^-20.
-                float upper = FLT_MAX;
+                // ---- the decision, every candidate in double (two bounded fp32 passes before it cost
+                // more: 64 channels x 576 lost 0.5 us a step to their barriers)
                 for (int g = gt; g < G; g += NT) {
-                    const float sh = fg(g) * smax_e;
-                    const float Nf = (float)(int)(Nbase + mN[g + 1]);
-                    const float Pf = i64_to_f32(Pbase + bin64(mLo, mHi, g + 1)) * pscale;
-                    const float D32 = sh * (sh * Nf - 2.0f * Pf);
-                    const float err = sh * (sh * Nf + 2.0f * Pf) * MPQ_FAST_REL;
-                    upper = fminf(upper, D32 + err);
-                }
-                upper = group_min<WPC>(upper, sc, gw, lane, grp);
-                for (int g = gt; g < G; g += NT) {
-                    const float sh = fg(g) * smax_e;
-                    const long long Pg = Pbase + bin64(mLo, mHi, g + 1);
-                    const long long Ng = Nbase + mN[g + 1];
-                    const float Nf = (float)(int)Ng;
-                    const float Pf = i64_to_f32(Pg) * pscale;
-                    const float D32 = sh * (sh * Nf - 2.0f * Pf);
-                    const float err = sh * (sh * Nf + 2.0f * Pf) * MPQ_FAST_REL;
-                    if (D32 - err <= upper) {
-                        const double D = decision(__fmul_rn(fg(g), smax), Pg, Ng, down);
-                        if (D < bestD) {
-                            bestD = D;
-                            bestg = g;
-                        }
+                    const double D = decision(__fmul_rn(fg(g), smax), Pbase + bin64(mLo, mHi, g + 1),
+                                              Nbase + mN[g + 1], down);
+                    if (D < bestD) {
+                        bestD = D;
+                        bestg = g;
                     }
                 }
             } else {
@@ -1204,7 +1179,7 @@ mpq_status launch_lat(bool lat, const float *W, int C, int d, int qmax, int G,
         if (lat) {
             // the lattice form on the linear grid: no grid table when that fits one more CTA on
             // an SM (it costs some arithmetic per candidate otherwise)
-            const size_t notab = smem - (size_t)2 * G * sizeof(float);
+            const size_t notab = smem - table_bytes(G);
             const int n_notab = quantize_ctas_per_sm<WPC, false, true, false>(notab);
             const int n_tab = quantize_ctas_per_sm<WPC, false, true, true>(smem);
             if constexpr (WPC == 4) {
@@ -1255,32 +1230,45 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
                        float *rmax, cudaStream_t stream)
 {
     const int hbits = ceil_log2((long long)d * qmax) + 1;
-    // lattice form on the linear grid when its buckets fit (32 KB) and their fields one word
+    const long long smem_cap = max_smem_optin();
+    // Lattice form on the linear grid when a bucket's fields fit one word, and the lattice is small
+    // or (its per-step cost is O(G Qmax), the event form's O(d) times the levels crossed) the row is
+    // long for it and it still fits: 64 x 576 with 8-bit codes and G = 64, 333 -> 80 us.
     LatBits lb;
-    const bool lat = !CUSTOM && (long long)2 * G * qmax + 1 <= 4096 && lattice_bits(d, qmax, G, &lb);
+    const long long nb_all = (long long)2 * G * qmax + 1;
+    bool lat = !CUSTOM && nb_all <= 40000 && lattice_bits(d, qmax, G, &lb);
+    if (lat) {
+        lb.nc = lattice_positions(G, qmax);
+        if (nb_all > 4096)
+            lat = G <= 2 * d && (long long)(group_words(G, d, 1, lb.nc) * 4 + table_bytes(G) +
+                                            lut_bytes((int)nb_all)) <= smem_cap;
+    }
     if (!lat) lb = LatBits{0, 31, 0};
-    const int nb = lat ? 2 * G * qmax + 1 : 0;
-    if (lat) lb.nc = lattice_positions(G, qmax);
+    const int nb = lat ? (int)nb_all : 0;
     const int nc = lb.nc;
     const size_t per_group = group_words(G, d, 1, nc) * 4;
-    const long long smem_cap = max_smem_optin();
-    // Warps per channel: enough channels in flight to fill the GPU, at least ~2 elements per
-    // lane, and enough warps per SM (24) for the shared memory the channels need -- on layers with
-    // thousands of long channels, 4-warp groups (more channels per SM, barriers over fewer warps)
-    // measured faster than 8-warp ones (c5's 11008 x 4096 layer: 2.28 -> 2.20 ms).
-    const long long warps_gpu = (long long)sm_count() * 32;
+    // Warps per channel.  A step's fixed work (scans, fold, decision, barriers) grows with the warps
+    // of a channel, so no more of them than fill the GPU to about 27 warps an SM (1280 x 320: 2
+    // warps 58 us, 4 warps 96), at least ~16 elements per warp (candidates, on rows evaluated
+    // directly), at least 4 warps for rows of 1,024 and more (4096 x 1024, G = 256: 200 us against
+    // 323 with 2), and enough warps per SM (24) for the shared memory the channels need -- on
+    // layers with thousands of long channels, 4-warp groups (more channels per SM, barriers over
+    // fewer warps) measured faster than 8-warp ones (11008 x 4096: 1.51 ms against 1.94).
+    const long long warps_gpu = (long long)sm_count() * 27;
     int wpc_c = 1;
-    while (wpc_c < 8 && (long long)C * wpc_c < warps_gpu) wpc_c *= 2;
+    while (wpc_c < 8 && (long long)C * wpc_c * 2 <= warps_gpu) wpc_c *= 2;
     int wpc_e = 1;
-    while (wpc_e < 8 && wpc_e * 64 <= d) wpc_e *= 2;
+    if (d <= QDIRECT_MAX_D) wpc_e = G >= 64 ? 2 : 1;
+    else
+        while (wpc_e < 8 && wpc_e * 16 <= d) wpc_e *= 2;
     const long long groups_per_sm = (long long)(227 * 1024) / (long long)(per_group + 256);
-    int wpc_s = 1;
+    int wpc_s = d >= 1024 ? 4 : 1;
     while (wpc_s < 8 && groups_per_sm * wpc_s < 24) wpc_s *= 2;
     int wpc = wpc_c < wpc_e ? wpc_c : wpc_e;
     if (wpc < wpc_s) wpc = wpc_s;
     for (; wpc <= 8; wpc *= 2) {
         const size_t smem = (size_t)(8 / wpc) * group_words(G, d, lat ? 1 : wpc, nc) * 4 +
-                            (size_t)2 * G * sizeof(float) + (lat ? lut_bytes(nb) : 0);
+                            table_bytes(G) + (lat ? lut_bytes(nb) : 0);
         if ((long long)smem <= smem_cap) {
             switch (wpc) {
             case 1:
