@@ -27,15 +27,16 @@
 // memory.  A thread of the epilogue holds one calibration row (TMEM lane) and 128 operand rows
 // (columns), so a channel's chain runs inside a thread.
 //
-// Schedule.  One resident pair per two SMs; `gang` neighbouring pairs share the row tiles of a
+// Schedule.  One resident pair per two SMs.  Either `gang` neighbouring pairs share the row tiles of a
 // channel tile and go through the same range of channel tiles, so its W and codes are read from
-// memory once for all of them (the pairs of a gang run at about the same pace).  Where a gang has
-// several pairs each leaves its sums of a tile in global scratch and the last one to arrive adds
-// them in pair order (nobody waits).  The gang size is the one with the least work on the
-// busiest pair, the larger on ties.  Measured on an 11008 x 4096 layer (N = 2048, k_max = 8): pairs
-// going through contiguous (channel tile, row tile) runs of their own 2.18 ms (each reads its W and
-// codes again for every row tile), gangs 2.08 ms; row tiles split over clusters of 2, 4 or 8 CTAs
-// 2.4 ms (whole waves of clusters, which do not fill the GPU's SM groups).
+// memory once for all of them (the pairs of a gang run at about the same pace); or every pair takes
+// an equal contiguous run of the (channel tile, row tile) units (gang 0), where that leaves less on
+// the busiest pair.  Where several pairs have a part of a channel tile, each leaves its sums in
+// global scratch and the last one to arrive adds them in pair order (nobody waits).  Measured on an
+// 11008 x 4096 layer (N = 2048, k_max = 8): contiguous runs 2.18 ms (each pair reads its W and codes
+// again for every row tile), gangs of four 2.08 ms; row tiles split over clusters of 2, 4 or 8 CTAs
+// 2.4 ms (whole waves of clusters, which do not fill the GPU's SM groups).  On 2009 x 432 (N = 636,
+// k_max = 8; 3.3 units a pair) gangs leave 6 units on a pair, contiguous runs 4: 54.8 -> XXX us.
 //
 // What bounds it: with the operand rows not written the same layer takes 2.02 ms, with W and codes
 // from one place of memory as well 1.77 ms, which is the MMAs alone (8 per step, 147 cycles each).
@@ -99,10 +100,10 @@ constexpr int E_MAX_XSLOTS = 4;
 constexpr int E_MAX_RAW = 4;
 constexpr uint32_t E_TMEM_COLS = 512;
 constexpr int E_MAX_PAIRS = 128;           // resident CTA pairs of a launch, at most
-constexpr int E_MAX_GANG = 8;              // pairs that share a channel tile's row tiles, at most
-// what the end of a channel tile costs its pair, and leaving its sums to a gang, in steps of 64
-// elements (about 0.6 us each on the tensor cores)
-constexpr int E_TILE_COST = 4, E_GANG_COST = 3;
+constexpr int E_MAX_GANG = 8;              // pairs that have a part of a channel tile, at most
+// what the end of a channel tile costs its pair, and leaving its sums to other pairs as well, in
+// steps of 64 elements (about 0.6 us each on the tensor cores)
+constexpr int E_TILE_COST = 1, E_PART_COST = 2;
 constexpr int E_SMEM_LIMIT = 232448;       // opt-in shared memory per CTA on sm_100 parts
 
 struct ChainCtrl {
@@ -119,7 +120,7 @@ struct ChainCtrl {
     uint32_t tmem_base;
     int abort;
     int xexp;
-    int last[2];                    // this CTA was the last of its gang to leave a tile's sums
+    int last[2];                    // this CTA was the last to leave a tile's sums
     float2 coef[E_N];               // per operand row of the pair: (2^{e_n - e_{n+1}}, s_n 2^e_n)
     int any_slow;                   // some channel of this CTA is left to slow_channel
     int slow[E_VEC];                // per channel of this CTA: 1 + the last pair tile where it is
@@ -331,11 +332,12 @@ __device__ __noinline__ void slow_channel(const float *__restrict__ X, int N, in
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void own_sync() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
 
-// Partial sums of a gang's pairs in global scratch, by channel tile and CTA of the pair: how many
-// pairs have arrived (zeroed before the launch), and E_VEC sums per pair.
+// Partial sums of the pairs that have a part of a channel tile, in global scratch, by tile and CTA of
+// the pair: how many have arrived (zeroed before the launch), and E_VEC sums per pair.
 struct ChainScratch {
     unsigned *count;   // [tiles][2]
-    double *slot;      // [tiles][gang][2][E_VEC]
+    double *slot;      // [tiles][parts][2][E_VEC]
+    int parts;
 };
 
 // scales: [C][k_max] point scales; xrange[0], vrange: max|X| and max|r| per residual vector, as
@@ -372,14 +374,30 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
     const int n_rt = (N + E_M - 1) / E_M;
     const int n_ks = (d + E_KS - 1) / E_KS;          // steps per row tile
     const int nseg = (n_ks + E_SEG - 1) / E_SEG;
-    // this pair's channel tiles [tile0, tile1) (its gang's) and row tiles [rt0, rt1) of each
-    const int n_gangs = (int)(gridDim.x >> 1) / gang;
-    const int gid = (int)(blockIdx.x >> 1) / gang, member = (int)(blockIdx.x >> 1) % gang;
-    const int tile0 = (int)((long long)tiles * gid / n_gangs);
-    const int tile1 = (int)((long long)tiles * (gid + 1) / n_gangs);
-    const int rt0 = (int)((long long)n_rt * member / gang);
-    const int rt1 = (int)((long long)n_rt * (member + 1) / gang);
-    const long long total = (long long)(tile1 - tile0) * (rt1 - rt0) * n_ks;
+    // this pair's channel tiles [tile0, tile1) and its row tiles of each: with a gang the same
+    // [rt0, rt1) of every one; else from rt0 on of the first and up to rt1 of the last
+    const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
+    int tile0, tile1, rt0, rt1, member = 0;
+    long long total;   // steps
+    if (gang > 0) {
+        const int n_gangs = n_pairs / gang, gid = pair / gang;
+        member = pair - gid * gang;
+        tile0 = (int)((long long)tiles * gid / n_gangs);
+        tile1 = (int)((long long)tiles * (gid + 1) / n_gangs);
+        rt0 = (int)((long long)n_rt * member / gang);
+        rt1 = (int)((long long)n_rt * (member + 1) / gang);
+        total = (long long)(tile1 - tile0) * (rt1 - rt0) * n_ks;
+    } else {
+        const long long units = (long long)tiles * n_rt;
+        const long long u0 = units * pair / n_pairs, u1 = units * (pair + 1) / n_pairs;
+        tile0 = (int)(u0 / n_rt);
+        tile1 = (int)((u1 - 1) / n_rt) + 1;
+        rt0 = (int)(u0 - (long long)tile0 * n_rt);
+        rt1 = (int)(u1 - (long long)(tile1 - 1) * n_rt);
+        total = (u1 - u0) * n_ks;
+    }
+    auto rt_lo = [&](int tile) { return gang > 0 || tile == tile0 ? rt0 : 0; };
+    auto rt_hi = [&](int tile) { return gang > 0 || tile == tile1 - 1 ? rt1 : n_rt; };
     // first channel of this CTA in a pair tile, and how many of its channels exist
     auto chan0 = [&](int tile) { return (tile * 2 + half) * CH; };
     auto n_chan = [&](int tile) { return max(0, min(CH, C - chan0(tile))); };
@@ -440,8 +458,9 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
             for (long long it = 0; it < total; ++it) {
                 if (left-- == 0) {
                     // a new tile's channels
-                    left = (long long)(rt1 - rt0) * n_ks - 1;
-                    nch = n_chan(++tile);
+                    ++tile;
+                    left = (long long)(rt_hi(tile) - rt_lo(tile)) * n_ks - 1;
+                    nch = n_chan(tile);
                     const int k0 = chan0(tile);
 #pragma unroll
                     for (int i = 0; i < G::ITEMS; ++i) {
@@ -541,9 +560,9 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                     }
                     if (++ks == n_ks) {
                         ks = 0;
-                        if (++rt == rt1) {
-                            rt = rt0;
+                        if (++rt == rt_hi(tile)) {
                             ++tile;
+                            rt = rt_lo(tile);
                         }
                     }
                     if (++rslot == RAW) {
@@ -697,7 +716,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
             slow = mine && mc < CH && ctl.slow[mc] == tile + 1;
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[i] = 0.0;
-            for (int rt = rt0; rt < rt1; ++rt) {
+            for (int rt = rt_lo(tile); rt < rt_hi(tile); ++rt) {
 #pragma unroll
                 for (int i = 0; i < E_VEC; ++i) sums[i] = 0.0f;
                 for (int sg = 0; sg < nseg; ++sg, ++g) {
@@ -773,21 +792,34 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                     note_timeout(wc, KBIT);
                     s = (double)NAN;
                 }
+                // which of the pairs that have a part of this tile this one is
+                int n_parts = gang, part_at = member;
+                if (gang == 0) {
+                    n_parts = 1;
+                    if (rt_lo(tile) > 0 || rt_hi(tile) < n_rt) {
+                        // (unit u is pair ((u + 1) n_pairs - 1) / units's)
+                        const long long units = (long long)tiles * n_rt, ut = (long long)tile * n_rt;
+                        const int p0 = (int)(((ut + 1) * n_pairs - 1) / units);
+                        n_parts = (int)(((ut + n_rt) * n_pairs - 1) / units) - p0 + 1;
+                        part_at = pair - p0;
+                    }
+                }
                 bool write = true;
-                if (gang > 1) {   // this pair's share into scratch; the last one adds them
-                    double *slots = part.slot + ((size_t)tile * gang * 2 + half) * E_VEC + m;
-                    slots[(size_t)member * 2 * E_VEC] = s;
+                if (n_parts > 1) {   // this pair's share into scratch; the last one adds them
+                    double *slots = part.slot + ((size_t)tile * part.parts * 2 + half) * E_VEC + m;
+                    slots[(size_t)part_at * 2 * E_VEC] = s;
                     __threadfence();
                     own_sync();
                     if (m == 0)
                         ctl.last[rb] = atomicAdd(part.count + 2 * (size_t)tile + half, 1u) ==
-                                       (unsigned)(gang - 1);
+                                       (unsigned)(n_parts - 1);
                     own_sync();
                     write = ctl.last[rb] != 0;
                     if (write) {
                         __threadfence();
                         s = 0.0;
-                        for (int p = 0; p < gang; ++p) s += __ldcg(slots + (size_t)p * 2 * E_VEC);
+                        for (int p = 0; p < n_parts; ++p)
+                            s += __ldcg(slots + (size_t)p * 2 * E_VEC);
                     }
                 }
                 const int k = chan0(tile) + mc;
@@ -805,8 +837,9 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
 
     cluster_sync();   // nothing of the pair's is in flight: the peer's sums have been read
     if (warp >= E_EPI_WARP0 && ctl.any_slow && !*abort_flag) {
-        // slow channels, by the gang's first pair
-        for (int tl = tile0; member == 0 && tl < tile1; ++tl) {
+        // slow channels, by the pair that has a tile's first row tile
+        for (int tl = tile0; tl < tile1; ++tl) {
+            if (rt_lo(tl) != 0) continue;
             for (int c = 0; c < n_chan(tl); ++c) {
                 const size_t k = (size_t)(chan0(tl) + c);
                 if (!is_slow<KP1>(vrange, scales, k)) continue;
@@ -890,25 +923,39 @@ mpq_status launch_chain(const float *X, const void *A, int N, const float *W, co
         pairs = std::max(1, std::min(pairs, E_MAX_PAIRS));
         resident.store(pairs, std::memory_order_relaxed);
     }
-    // the gang size (see the top), within the scratch given
-    int gang = 1;
+    // the schedule with the least work on the busiest pair (see the top) within the scratch given;
+    // on ties the larger gang, contiguous runs only where they are better
+    int gang = 1, parts = 1;
     long long best = -1;
     for (int g = 1; g <= E_MAX_GANG && g <= n_rt && g <= pairs; g *= 2) {
         const long long gangs = std::min<long long>(pairs / g, tiles);
         const long long cost = ((tiles + gangs - 1) / gangs) *
                                ((long long)((n_rt + g - 1) / g) * n_ks + E_TILE_COST +
-                                (g > 1 ? E_GANG_COST : 0));
+                                (g > 1 ? E_PART_COST : 0));
         if (g > 1 && chain_scratch_bytes(tiles, g) > part_bytes) break;
         if (best < 0 || cost <= best) {
             best = cost;
             gang = g;
+            parts = g;
         }
     }
-    pairs = (int)std::min<long long>(pairs / gang, tiles) * gang;
+    const long long units = (long long)tiles * n_rt;
+    const long long runs = std::min<long long>(pairs, units);        // pairs with a run of their own
+    const long long most = (units + runs - 1) / runs, least = units / runs;
+    const long long split = std::min<long long>(n_rt, (n_rt + 2 * least - 2) / least);   // of a tile
+    const long long over = std::min<long long>(most, (most + 2LL * n_rt - 2) / n_rt);    // tiles of a run
+    const double reread = (double)C * d * (4 + G::K) > 64e6 ? 1.06 : 1.0;   // W and codes beyond L2
+    if (split <= E_MAX_GANG && chain_scratch_bytes(tiles, (int)split) <= part_bytes &&
+        reread * (double)(most * n_ks + over * (E_TILE_COST + E_PART_COST)) < (double)best) {
+        gang = 0;
+        parts = (int)split;
+    }
+    pairs = gang > 0 ? (int)std::min<long long>(pairs / gang, tiles) * gang : (int)runs;
     cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
     ChainScratch sp;
     sp.count = static_cast<unsigned *>(part);
     sp.slot = reinterpret_cast<double *>(static_cast<char *>(part) + chain_count_bytes(tiles));
+    sp.parts = parts;
     WaitCtl wc;
     const mpq_status wst = wait_ctl(&wc);
     if (wst != MPQ_OK) return wst;
