@@ -311,10 +311,8 @@ mpq_status launch_allocate_budget(const float *err, int C, int k_max, long long 
     const long long nkeys = (long long)C * (k_max - 1);
     const bool cached = nkeys <= KEY_CACHE;
     const size_t smem = cached ? (size_t)nkeys * sizeof(unsigned) : 0;
-    // always the same limit: calls of other threads may come between this and the launch
-    cudaError_t e = cudaFuncSetAttribute(allocate_budget_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         KEY_CACHE * (int)sizeof(unsigned));
+    static std::atomic<int> limit[kMaxDevices];
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(allocate_budget_kernel), limit, smem);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
     allocate_budget_kernel<<<1, AB_THREADS, smem, stream>>>(err, C, k_max, extra, npoints,
                                                             points_used, cached);
@@ -350,9 +348,8 @@ mpq_status launch_allocate_batch(int n, const float *const *err, const int *C, i
             b.order[j] = b.order[j - 1];
             b.order[j - 1] = t;
         }
-    const cudaError_t e = cudaFuncSetAttribute(allocate_batch_kernel,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               KEY_CACHE * (int)sizeof(unsigned));
+    static std::atomic<int> limit[kMaxDevices];
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(allocate_batch_kernel), limit, smem);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
     allocate_batch_kernel<<<m, AB_THREADS, smem, stream>>>(b, k_max, mode);
     return cuda_status(cudaGetLastError(), "batched allocation kernel launch");

@@ -58,6 +58,24 @@ int max_smem_optin()
     return cache[dev];
 }
 
+cudaError_t allow_smem(const void *kernel, std::atomic<int> (&limit)[kMaxDevices], size_t bytes)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool kept = dev >= 0 && dev < kMaxDevices;
+    const int have = kept ? limit[dev].load(std::memory_order_relaxed) : 0;
+    if (have > 0 && (size_t)have >= bytes) return cudaSuccess;
+    cudaFuncAttributes at;
+    e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess) return e;
+    const int left = max_smem_optin() - (int)at.sharedSizeBytes;
+    if (left < 0 || bytes > (size_t)left) return cudaErrorInvalidValue;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, left);
+    if (e == cudaSuccess && kept) limit[dev].store(left, std::memory_order_relaxed);
+    return e;
+}
+
 }  // namespace mpq
 
 using namespace mpq;

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "checks.cuh"
 #include "mpq.h"
 
@@ -43,6 +45,11 @@ int sm_count();
 
 // Opt-in dynamic shared memory limit per block of the current device (cached per device).
 int max_smem_optin();
+
+// Raises a kernel's dynamic shared memory limit to all its device has left, once per device (`limit`
+// holds what was set, 0 at first): launches of other threads with other sizes then never find it
+// lowered, and later calls cost no runtime call.
+cudaError_t allow_smem(const void *kernel, std::atomic<int> (&limit)[kMaxDevices], size_t bytes);
 
 struct GridFrac {
     float f[MPQ_MAX_GRID];

@@ -747,8 +747,8 @@ mpq_status launch_mma(const int8_t *X, int T, const mpq_packed_layout *L, const 
     const bool aligned = L->d % 8 == 0 && (uintptr_t)X % 8 == 0;
     auto kernel = aligned ? multipoint_mma_kernel<MT, NT, true> : multipoint_mma_kernel<MT, NT, false>;
     const int smem = (int)sizeof(int) * S_WARPS * 16 * MT * 8 * NT;
-    const cudaError_t e =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static std::atomic<int> limit[2][kMaxDevices];
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kernel), limit[aligned], smem);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
     const long long n_blocks = ((long long)T + 8 * NT - 1) / (8 * NT);
     const long long blocks = n_blocks * (L->rows / (16 * MT));
@@ -926,8 +926,9 @@ mpq_status launch_multipoint_linear(const int8_t *X, int T, const mpq_packed_lay
             set_error("multipoint linear needs %d bytes of shared memory", L_SMEM);
             return MPQ_ERR_UNSUPPORTED;
         }
-        const cudaError_t e = cudaFuncSetAttribute(
-            multipoint_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L_SMEM);
+        static std::atomic<int> limit[kMaxDevices];
+        const cudaError_t e =
+            allow_smem(reinterpret_cast<const void *>(multipoint_linear_kernel), limit, L_SMEM);
         if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
         WaitCtl wc;
         const mpq_status wst = wait_ctl(&wc);

@@ -36,7 +36,7 @@
 // 11008 x 4096 layer (N = 2048, k_max = 8): contiguous runs 2.18 ms (each pair reads its W and codes
 // again for every row tile), gangs of four 2.08 ms; row tiles split over clusters of 2, 4 or 8 CTAs
 // 2.4 ms (whole waves of clusters, which do not fill the GPU's SM groups).  On 2009 x 432 (N = 636,
-// k_max = 8; 3.3 units a pair) gangs leave 6 units on a pair, contiguous runs 4: 54.8 -> XXX us.
+// k_max = 8; 3.3 units a pair) gangs leave 6 units on a pair, contiguous runs 4.
 //
 // What bounds it: with the operand rows not written the same layer takes 2.02 ms, with W and codes
 // from one place of memory as well 1.77 ms, which is the MMAs alone (8 per step, 147 cycles each).
@@ -48,8 +48,8 @@
 // (lane 0 of the even CTA), 8-15 the epilogue (lane quarter warp % 4, column half).  Steps of 64
 // elements: X tiles land straight in their slots (split ahead into fp16 planes), W and codes in a
 // ring that the producers read.  RAWX (the entry point with fixed scratch): X lands unsplit in that
-// ring, and the producers and, between their folds, the epilogue warps split it; same operands, same MMAs in the same order, so the results
-// are bit-identical.  Every wait is bounded; on a timeout the kernel records
+// ring, and the producers and, between their folds, the epilogue warps split it; same operands, same
+// MMAs in the same order, so the results are bit-identical.  Every wait is bounded; on a timeout the kernel records
 // MPQ_TIMEOUT_OUTPUT_ERROR, waits for what it issued, and the outputs read NaN.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -85,8 +85,8 @@ constexpr int E_MMA_WARP = 7;
 constexpr int E_EPI_WARP0 = 8;             // a multiple of 4: warp % 4 is the TMEM lane quarter
 constexpr int E_EPI_WARPS = 8;
 constexpr int E_THREADS = 512;
-// RAWX: X items of a step split by the epilogue warps (c5's up_proj 3.79 ms, c3's 512 x 4608 237 us;
-// none: 4.07 and 271, 6 * 256: 4.20 and 209)
+// RAWX: X items of a step split by the epilogue warps (11008 x 4096 3.79 ms, 512 x 4608 237 us; none:
+// 4.07 and 271, 6 * 256: 4.20 and 209)
 constexpr int E_X_EPI = 4 * 256;
 // registers per thread after setmaxnreg: warpgroups 0-1 and 2-3 (epilogue); together exactly what
 // the launch holds (512 threads x 128)
@@ -898,8 +898,9 @@ mpq_status launch_chain(const float *X, const void *A, int N, const float *W, co
         set_error("output error needs %d bytes of shared memory", G::SMEM);
         return MPQ_ERR_UNSUPPORTED;
     }
-    cudaError_t e = cudaFuncSetAttribute(output_error_chain_kernel<KP1, RAWX>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+    static std::atomic<int> limit[kMaxDevices];
+    cudaError_t e = allow_smem(reinterpret_cast<const void *>(output_error_chain_kernel<KP1, RAWX>),
+                               limit, G::SMEM);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
 
     cudaLaunchConfig_t cfg = {};

@@ -1116,6 +1116,12 @@ struct LatBits {
 
 int lattice_positions(int G, int qmax)
 {
+    // counted once per (G, Qmax) and kept in a small table (key and count in one word)
+    static std::atomic<unsigned long long> table[64];
+    const unsigned key = (unsigned)G << 8 | (unsigned)qmax;
+    std::atomic<unsigned long long> &at = table[(key ^ key >> 6 ^ key >> 12) & 63u];
+    const unsigned long long kept = at.load(std::memory_order_relaxed);
+    if ((unsigned)(kept >> 32) == key) return (int)(unsigned)kept;
     std::vector<char> seen((size_t)2 * G * qmax + 1, 0);
     int n = 0;
     for (int g = 1; g <= G; ++g)
@@ -1126,6 +1132,7 @@ int lattice_positions(int G, int qmax)
                 ++n;
             }
         }
+    at.store((unsigned long long)key << 32 | (unsigned)n, std::memory_order_relaxed);
     return n;
 }
 
@@ -1144,8 +1151,9 @@ mpq_status launch_wpc(const float *W, int C, int d, int qmax, int G, const Grid<
                       float *rmax, int hbits, LatBits lb, size_t smem, cudaStream_t stream)
 {
     constexpr int GPC = 8 / WPC;
-    cudaError_t e = cudaFuncSetAttribute(quantize_kernel<WPC, CUSTOM, LAT, TABLE, MINB, TM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<int> limit[kMaxDevices];
+    cudaError_t e = allow_smem(
+        reinterpret_cast<const void *>(quantize_kernel<WPC, CUSTOM, LAT, TABLE, MINB, TM>), limit, smem);
     if (e == cudaSuccess) {
         quantize_kernel<WPC, CUSTOM, LAT, TABLE, MINB, TM><<<(C + GPC - 1) / GPC, QTHREADS, smem, stream>>>(
             W, C, d, qmax, G, grid, k_max, codes, scales, resid_sq, residuals, rmax, hbits, lb.lat_bits,
@@ -1155,17 +1163,23 @@ mpq_status launch_wpc(const float *W, int C, int d, int qmax, int G, const Grid<
     return cuda_status(e, "quantize kernel launch");
 }
 
-// CTAs of a quantize kernel that fit on one SM with `smem` bytes of dynamic shared memory.
+// CTAs of a quantize kernel that fit on one SM with `smem` bytes of dynamic shared memory (the last
+// answer of each kernel is kept: one size and its count in a word; one kind of device per process).
 template <int WPC, bool CUSTOM, bool LAT, bool TABLE, int MINB = 4, bool TM = false>
 int quantize_ctas_per_sm(size_t smem)
 {
+    static std::atomic<unsigned long long> last{0};
+    const unsigned long long seen = last.load(std::memory_order_relaxed);
+    if (seen != 0 && (seen >> 8) == smem) return (int)(seen & 255u) - 1;
+    static std::atomic<int> limit[kMaxDevices];
     int n = 0;
-    if (cudaFuncSetAttribute(quantize_kernel<WPC, CUSTOM, LAT, TABLE, MINB, TM>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(reinterpret_cast<const void *>(quantize_kernel<WPC, CUSTOM, LAT, TABLE, MINB, TM>),
+                   limit, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, quantize_kernel<WPC, CUSTOM, LAT, TABLE, MINB, TM>,
                                                       QTHREADS, smem) != cudaSuccess)
         n = 0;
     (void)cudaGetLastError();
+    last.store(((unsigned long long)smem << 8) | (unsigned)(n + 1), std::memory_order_relaxed);
     return n;
 }
 
