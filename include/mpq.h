@@ -124,12 +124,14 @@ mpq_status mpq_quantize_layer(const float *W, int C, int d, int bits, int G,
  * Scratch: with groups == 1, d a multiple of 16 and X, W, codes 16-byte aligned (the tensor-core
  * path with scaled fp16 operands), the call takes 4 (1 + C (k_max+1)) bytes (4 bytes with rmax),
  * rounded up to 256, plus 4 N d bytes for X's fp16 hi/lo planes, plus partial sums: 8 + 16384 bytes
- * per tile of 2 floor(128 / (k_max + 2)) channels (8 bytes where N <= 256)
- * from the current device's default stream-ordered memory pool with cudaMallocAsync on `stream`
+ * per tile of 2 floor(128 / (k_max + 2)) channels (8 bytes where N <= 256; 4 MiB at most) from the current device's default stream-ordered memory pool with cudaMallocAsync on `stream`
  * and returns them with cudaFreeAsync on `stream` -- concurrent calls on other streams each get
  * their own, and a CUDA graph capture records them as the graph's allocation nodes.
- * MPQ_ERR_NOMEM if that allocation fails (nothing else is enqueued then).  The first such call in
- * a process made outside a stream capture raises that pool's release threshold
+ * MPQ_ERR_NOMEM if that allocation fails (nothing else is enqueued then).  Other rows (groups ==
+ * 1) from 192 elements on, with at least 256 / (k_max + 2) channels (or from 600 on with k_max >= 4),
+ * take the same with d rounded up to 16, plus (4 + k_max) C d bytes so rounded for copies of W and
+ * the codes; if the pool has no room for that, a kernel without scratch computes them (equal within
+ * rounding).  The first such call in a process made outside a stream capture raises that pool's release threshold
  * (cudaMemPoolAttrReleaseThreshold) to keep freed blocks cached in the pool instead of returning
  * them to the driver at every synchronization; a process that manages the default pool itself
  * can call mpq_output_error_noalloc instead.

@@ -17,6 +17,8 @@ namespace mpq {
 
 static thread_local char g_msg[512];
 
+void clear_error() { g_msg[0] = 0; }
+
 void set_error(const char *fmt, ...)
 {
     va_list ap;
@@ -241,7 +243,7 @@ extern "C" mpq_status mpq_output_error_noalloc(const float *X, int N, int groups
     g_msg[0] = 0;
     const mpq_status st = check_output_error(X, N, groups, W, codes, scales, C, d, k_max, err);
     if (st != MPQ_OK || C == 0) return st;
-    const size_t words = output_error_scratch_words(X, groups, W, codes, C, d, k_max);
+    const size_t words = output_error_scratch_words(X, N, groups, W, codes, C, d, k_max);
     REQUIRE(words <= (size_t)MPQ_NOALLOC_RANGE_WORDS, MPQ_ERR_UNSUPPORTED,
             "C = %d, k_max = %d need %zu scratch words; the fixed buffer holds %d", C, k_max, words,
             MPQ_NOALLOC_RANGE_WORDS);

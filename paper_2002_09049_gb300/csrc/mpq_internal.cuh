@@ -30,8 +30,10 @@ __device__ __forceinline__ float mean_of_sum(float sum, int N)
 }
 
 
-// Records a formatted failure message for mpq_last_error() on the calling thread.
+// Records a formatted failure message for mpq_last_error() on the calling thread; clear_error
+// forgets it (a failure that another path makes good).
 void set_error(const char *fmt, ...);
+void clear_error();
 
 // Maps a CUDA error to MPQ_ERR_CUDA (recording its text), cudaSuccess to MPQ_OK.
 mpq_status cuda_status(cudaError_t e, const char *what);
@@ -73,15 +75,17 @@ mpq_status launch_output_error(const float *X, int N, int groups, const float *W
 // (larger layers leave each channel tile to one CTA pair).
 constexpr size_t CHAIN_FIXED_SCRATCH = 1 << 22;
 // Words of range scratch a call needs (0 where it takes no scratch).
-size_t output_error_scratch_words(const float *X, int groups, const float *W,
+size_t output_error_scratch_words(const float *X, int N, int groups, const float *W,
                                   const int8_t *codes, int C, int d, int k_max);
 
 mpq_status launch_output_error_tc(const float *X, int N, const float *W, const int8_t *codes,
                                   const float *scales, int C, int d, int k_max, float *err,
                                   cudaStream_t stream);
 
-// CTA-pair tensor-core kernel: needs d % 16 == 0 and 16-byte aligned X, W and codes.
+// CTA-pair tensor-core kernel: with d % 16 == 0 and 16-byte aligned X, W and codes it reads them
+// with tile copies (pair_ok); other rows it gathers or reads from padded copies, where rows_ok.
 bool output_error_pair_ok(const float *X, const float *W, const int8_t *codes, int d);
+bool output_error_rows_ok(int N, const int8_t *codes, int C, int d, int k_max);
 mpq_status launch_output_error_pair(const float *X, int N, const float *W, const int8_t *codes,
                                     const float *scales, int C, int d, int k_max, float *err,
                                     cudaStream_t stream, unsigned *range, const float *rmax);

@@ -133,10 +133,13 @@ mpq_status launch_grouped(const float *X, int N, const float *W, const int8_t *c
 
 }  // namespace
 
-size_t output_error_scratch_words(const float *X, int groups, const float *W,
+size_t output_error_scratch_words(const float *X, int N, int groups, const float *W,
                                   const int8_t *codes, int C, int d, int k_max)
 {
-    return (groups == 1 && output_error_pair_ok(X, W, codes, d)) ? 1 + (size_t)C * (k_max + 1) : 0;
+    return (groups == 1 && (output_error_pair_ok(X, W, codes, d) ||
+                            output_error_rows_ok(N, codes, C, d, k_max)))
+               ? 1 + (size_t)C * (k_max + 1)
+               : 0;
 }
 
 mpq_status launch_output_error(const float *X, int N, int groups, const float *W,
@@ -148,6 +151,12 @@ mpq_status launch_output_error(const float *X, int N, int groups, const float *W
         if (output_error_pair_ok(X, W, codes, d))
             return launch_output_error_pair(X, N, W, codes, scales, C, d, k_max, err, stream,
                                             range, rmax);
+        if (output_error_rows_ok(N, codes, C, d, k_max)) {
+            const mpq_status st = launch_output_error_pair(X, N, W, codes, scales, C, d, k_max, err,
+                                                           stream, range, rmax);
+            if (st != MPQ_ERR_NOMEM) return st;   // nothing enqueued: the kernel without scratch
+            clear_error();
+        }
         return launch_output_error_tc(X, N, W, codes, scales, C, d, k_max, err, stream);
     }
     switch (k_max + 1) {

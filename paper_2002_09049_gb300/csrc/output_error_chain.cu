@@ -104,6 +104,9 @@ constexpr int E_MAX_GANG = 8;              // pairs that have a part of a channe
 // what the end of a channel tile costs its pair, and leaving its sums to other pairs as well, in
 // steps of 64 elements (about 0.6 us each on the tensor cores)
 constexpr int E_TILE_COST = 1, E_PART_COST = 2;
+constexpr int E_GATHERERS = E_PROD_WARPS + 1;
+// bytes of a gathered row of X or W, and of codes: 64 elements from any offset into 16 bytes
+constexpr int E_GATHER_F = E_KS * 4 + 16, E_GATHER_Q = E_KS + 16;
 constexpr int E_SMEM_LIMIT = 232448;       // opt-in shared memory per CTA on sm_100 parts
 
 struct ChainCtrl {
@@ -131,18 +134,21 @@ constexpr int E_CTRL_BYTES = (sizeof(ChainCtrl) + 1023) / 1024 * 1024;
 constexpr int E_BASE_SMEM = 1024 /* alignment slack */ + E_CTRL_BYTES;
 
 // Per-k_max geometry.  Raw slot, as the tile copies write it: W step [CH][64] fp32, codes
-// [K][CH][64] int8, and (RAWX) X step [128][64] fp32 first.  X slots: as many as leave room for
-// three operand stages and at least two raw slots.
+// [K][CH][64] int8, and (RAWX) X step [128][64] fp32 first; a gathered slot's rows are
+// E_GATHER_F or E_GATHER_Q bytes.  X slots: as many as leave room for three operand
+// stages and at least two raw slots.
 template <int KP1, bool RAWX>
 struct EGeo {
     static constexpr int K = KP1 - 1;
     static constexpr int R = KP1 + 1;                    // operand rows per channel
     static constexpr int CH = E_VEC / R;                 // channels per CTA
     static constexpr int ITEMS = (CH * 16 + E_PT - 1) / E_PT;   // 16 items of 4 elements per channel
-    static constexpr int RAW_W = RAWX ? E_ROWS * E_KS * 4 : 0;
-    static constexpr int RAW_Q = RAW_W + CH * E_KS * 4;
-    static constexpr uint32_t RAW_TX = RAW_Q + K * CH * E_KS;
-    static constexpr int RAW_BYTES = (RAW_Q + K * CH * E_KS + 1023) / 1024 * 1024;
+    static constexpr int F_ROW = RAWX ? E_GATHER_F : E_KS * 4;   // reserved for a row
+    static constexpr int RAW_W = RAWX ? E_ROWS * F_ROW : 0;
+    static constexpr int RAW_Q = (RAW_W + CH * F_ROW + 127) / 128 * 128;
+    static constexpr uint32_t RAW_TX = ((RAWX ? E_ROWS : 0) + CH) * E_KS * 4 + K * CH * E_KS;
+    static constexpr int RAW_BYTES =
+        (RAW_Q + K * CH * (RAWX ? E_GATHER_Q : E_KS) + 1023) / 1024 * 1024;
     static constexpr int NS = RAWX ? 2 : 3;              // operand stages
     // RAWX: the producers write X's tiles beside the operand rows, stage by stage
     static constexpr int NX =
@@ -169,12 +175,27 @@ __device__ __forceinline__ void codes_f16x4(uint32_t biased, uint32_t &c01, uint
     c23 = *reinterpret_cast<const uint32_t *>(&y);
 }
 
+// 16 bytes of a gathered row, from any word.
+__device__ __forceinline__ float4 ld_gathered(uint32_t a)
+{
+    float4 v;
+    v.x = __uint_as_float(ld_shared_u32(a));
+    v.y = __uint_as_float(ld_shared_u32(a + 4u));
+    v.z = __uint_as_float(ld_shared_u32(a + 8u));
+    v.w = __uint_as_float(ld_shared_u32(a + 12u));
+    return v;
+}
+
 // Raw slot -> the operand rows of one step (tile `dst`): for every (channel, 4 contiguous
 // elements) item the codes of every point as fp16, then the last residual (Eq. 7's recursion in
 // fp32) scaled by 2^e and split into hi and lo.  Every shared-memory read before the stores; a
-// half warp's 8-byte stores fill one 128-byte row.
+// half warp's 8-byte stores fill one 128-byte row.  gather: the slot's rows are the aligned 16 bytes
+// around the elements; w0: address of W's row of the CTA's first channel, q0 of its codes of point 1,
+// d: row length, plane: codes of a point (all of these count by their low four bits only, and a
+// step starts a multiple of 64 elements into the row).
 template <int KP1, bool RAWX>
-__device__ __forceinline__ void chain_rows(uint32_t slot, uint32_t dst, int pt, int nch,
+__device__ __forceinline__ void chain_rows(uint32_t slot, uint32_t dst, int pt, int nch, bool gather,
+                                           uint32_t w0, uint32_t q0, uint32_t d, uint32_t plane,
                                            const float (&sc)[EGeo<KP1, RAWX>::ITEMS][KP1 - 1],
                                            const float (&vf)[EGeo<KP1, RAWX>::ITEMS])
 {
@@ -185,12 +206,26 @@ __device__ __forceinline__ void chain_rows(uint32_t slot, uint32_t dst, int pt, 
         const int p = pt + i * E_PT;
         if (p < nch * 16) {
             const int ch = p >> 4, e4 = p & 15;
-            float4 r = ld_shared_v4(slot + G::RAW_W + (uint32_t)(ch * E_KS + e4 * 4) * 4u);
+            float4 r;
+            if (RAWX && gather)
+                r = ld_gathered(slot + G::RAW_W + (uint32_t)(ch * E_GATHER_F + e4 * 16) +
+                                ((w0 + (uint32_t)ch * d * 4u) & 15u));
+            else
+                r = ld_shared_v4(slot + G::RAW_W + (uint32_t)(ch * E_KS + e4 * 4) * 4u);
             uint32_t qb[K];
 #pragma unroll
-            for (int n = 0; n < K; ++n)
-                qb[n] = ld_shared_u32(slot + G::RAW_Q + (uint32_t)((n * G::CH + ch) * E_KS + e4 * 4)) ^
-                        0x80808080u;
+            for (int n = 0; n < K; ++n) {
+                if (RAWX && gather) {
+                    const uint32_t at = q0 + (uint32_t)n * plane + (uint32_t)ch * d;
+                    const uint32_t a = slot + G::RAW_Q + (at & 12u) +
+                                       (uint32_t)((n * G::CH + ch) * E_GATHER_Q + e4 * 4);
+                    qb[n] = __funnelshift_r(ld_shared_u32(a), ld_shared_u32(a + 4u), 8u * (at & 3u));
+                } else {
+                    qb[n] = ld_shared_u32(slot + G::RAW_Q +
+                                          (uint32_t)((n * G::CH + ch) * E_KS + e4 * 4));
+                }
+                qb[n] ^= 0x80808080u;
+            }
             const uint32_t cofs = (uint32_t)(e4 & 1) * 8u;   // 4 elements = 8 bytes of a 16-byte chunk
             const int row = ch * G::R;
 #pragma unroll
@@ -215,15 +250,22 @@ __device__ __forceinline__ void chain_rows(uint32_t slot, uint32_t dst, int pt, 
 
 // RAWX: items [p0, p1) of the step's X rows (row p / 16, 4 elements), `stride` threads apart, scaled
 // by 2^e and split into the hi and lo tiles (the same values as f16_split_kernel's planes).
+// gather: the slot's rows are the aligned 16 bytes around the elements, x0 the address of X and d the
+// row length, by their low bits (a row tile starts a multiple of 128 rows into X).
 template <int U>
 __device__ __forceinline__ void chain_x(uint32_t slot, uint32_t xset, int p0, int p1, int stride,
-                                        float xs)
+                                        float xs, bool gather, uint32_t x0, uint32_t d)
 {
     for (; p0 < p1; p0 += U * stride) {   // U reads in flight, all before their stores
         float4 x[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (p0 + u * stride < p1) x[u] = ld_shared_v4(slot + (uint32_t)(p0 + u * stride) * 16u);
+            if (const int p = p0 + u * stride; p < p1) {
+                const uint32_t row = (uint32_t)p >> 4;
+                x[u] = gather ? ld_gathered(slot + row * E_GATHER_F + ((uint32_t)p & 15u) * 16u +
+                                            ((x0 + row * d * 4u) & 15u))
+                              : ld_shared_v4(slot + (uint32_t)p * 16u);
+            }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int p = p0 + u * stride, row = p >> 4, e4 = p & 15;
@@ -258,6 +300,64 @@ __device__ __forceinline__ bool is_slow(const unsigned *__restrict__ vrange,
         vr = vn;
     }
     return slow;
+}
+
+// RAWX, rows that a tile copy cannot address: the producer warps and the copy warp each copy a share
+// (part 0 .. E_GATHERERS - 1) of the raw slot of a step (columns x .. x + 63, X rows row0 .. + 127,
+// channels k0 .. + nch - 1), for every row the aligned 16 bytes that hold its 64 elements, and arrive
+// on `bar` with every lane.  Zeros from the row's end on and outside the arrays; what lies before
+// the first element is not used.  No read outside an array: at its start, where the aligned 16
+// bytes may begin before it, the words inside are copied one by one (X, W and codes are 4-byte
+// aligned); at a row's end a copy reads no further.  (5245 x 1859, k_max = 5, N = 939: 1.12 ms; 4
+// bytes at a time 1.55 ms, and all by one warp 3.0 ms.)
+template <int PIECES>   // of 16 bytes, of which the last only where the row's offset needs it
+__device__ __forceinline__ void gather_rows(uint32_t dst, uintptr_t base, uintptr_t row0,
+                                            uint32_t row_bytes, uint32_t xb, int n, int valid, int th)
+{
+    constexpr int STEP = E_GATHERERS * 32 / PIECES;   // rows a pass; the threads left over idle
+    int r = th / PIECES;
+    const int c = th - r * PIECES;
+    if (r >= STEP) return;
+    uintptr_t at = row0 + (size_t)r * row_bytes + xb;
+    dst += (uint32_t)th * 16u;
+#pragma unroll 2
+    for (; r < n; r += STEP, at += (size_t)STEP * row_bytes, dst += STEP * PIECES * 16u) {
+        const int off = (int)(at & 15);
+        const uintptr_t from = at - (unsigned)off + 16u * (unsigned)c;
+        const int left = (int)(row_bytes - xb) + off - 16 * c;
+        const bool need = r < valid && (c < PIECES - 1 || off);
+        const uint32_t bytes = need ? (uint32_t)max(0, min(16, left)) : 0u;
+        if (bytes && from < base) {
+#pragma unroll 1
+            for (uint32_t o = (uint32_t)(base - from); o < 16u; o += 4u) {
+                const uint32_t b = o < bytes ? min(4u, bytes - o) : 0u;
+                cp_async4(dst + o, reinterpret_cast<const void *>(b ? from + o : base), b);
+            }
+        } else {
+            cp_async16(dst, reinterpret_cast<const void *>(bytes ? from : base & ~(uintptr_t)15),
+                       bytes);
+        }
+    }
+}
+
+template <int KP1>
+__device__ __noinline__ void gather_slot(int part, uint32_t slot, const float *__restrict__ X, int N,
+                                         const float *__restrict__ W,
+                                         const int8_t *__restrict__ codes, int C, int d, int x,
+                                         int row0, int k0, int nch, int lane, uint64_t *bar)
+{
+    using G = EGeo<KP1, true>;
+    const uintptr_t xp = (uintptr_t)X, wp = (uintptr_t)W, qp = (uintptr_t)codes;
+    const uint32_t fb = (uint32_t)d * 4u, xb = (uint32_t)x * 4u;
+    const int th = part * 32 + lane;
+    gather_rows<E_GATHER_F / 16>(slot, xp, xp + (size_t)row0 * fb, fb, xb, E_ROWS, N - row0, th);
+    gather_rows<E_GATHER_F / 16>(slot + G::RAW_W, wp, wp + (size_t)k0 * fb, fb, xb, nch, nch, th);
+#pragma unroll 1
+    for (int n = 0; n < G::K; ++n)
+        gather_rows<E_GATHER_Q / 16>(slot + G::RAW_Q + (uint32_t)(n * G::CH * E_GATHER_Q), qp,
+                                     qp + ((size_t)n * C + (size_t)k0) * d, (uint32_t)d, (uint32_t)x,
+                                     nch, nch, th);
+    cp_async_arrive(bar);
 }
 
 // Sum over the warp's 32 lanes of each of 32 values: lane l returns the sum of v[l].  Each exchange
@@ -368,6 +468,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
     const uint32_t ring_u32 = v_u32 + NS * E_TILE;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool gather = RAWX && !tile_rows_ok(X, W, codes, d);
     const uint32_t crank = cluster_ctarank();
     const int half = (int)crank;                     // 0: even CTA (issues the MMAs), 1: its peer
     const uint16_t pair_mask = 3u;
@@ -417,7 +518,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
             mbar_init(&ctl.xempty[s], 1);
         }
         for (int r = 0; r < RAW; ++r) {
-            mbar_init(&ctl.raw_full[r], 1);
+            mbar_init(&ctl.raw_full[r], gather ? E_GATHERERS * 32 : 1);   // who copies the slot
             mbar_init(&ctl.raw_empty[r], SPLIT_WARPS);
         }
         for (int b = 0; b < 2; ++b) {
@@ -441,6 +542,40 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
     const uint32_t tmem = ctl.tmem_base;
     volatile int *abort_flag = &ctl.abort;
 
+    // RAWX with gathered rows, by every warp of the producers and the copy warp: this warp's share of
+    // the steps before `upto`, each once its slot is free (false: give up; warp-uniform)
+    long long gf = 0;
+    int gks = 0, grt = rt0, gtile = tile0, gslot = 0;
+    uint32_t gph = 1;
+    auto gather_to = [&](long long upto) -> bool {
+        for (; gf < upto && gf < total; ++gf) {
+            bool ok = !*abort_flag;
+            if (ok && gf >= RAW) {
+                ok = mbar_wait(&ctl.raw_empty[gslot], gph, wc.budget);
+                if (!ok) note_timeout(wc, KBIT);
+            }
+            if (__any_sync(0xffffffffu, !ok)) {
+                *abort_flag = 1;
+                return false;
+            }
+            gather_slot<KP1>(warp, ring_u32 + gslot * G::RAW_BYTES, X, N, W, codes, C, d, gks * E_KS,
+                             grt * E_M + half * E_ROWS, chan0(gtile), n_chan(gtile), lane,
+                             &ctl.raw_full[gslot]);
+            if (++gks == n_ks) {
+                gks = 0;
+                if (++grt == rt_hi(gtile)) {
+                    ++gtile;
+                    grt = rt_lo(gtile);
+                }
+            }
+            if (++gslot == RAW) {
+                gslot = 0;
+                gph ^= 1u;
+            }
+        }
+        return true;
+    };
+
     // one setmaxnreg per warpgroup: 0-1 give registers to 2-3 (epilogue)
     if (warp < E_EPI_WARP0) {
         setmaxnreg_dec<E_REGS_LOW>();
@@ -454,14 +589,14 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
             int s = 0, slot = 0, sx = 0;
             uint32_t sph = 0, rph = 0, xph = 0;    // phase parities of stage s, raw slot, X slot sx
             long long left = 0;         // steps left in the tile
-            int tile = tile0 - 1;
+            int tile = tile0 - 1, k0 = 0;
             for (long long it = 0; it < total; ++it) {
                 if (left-- == 0) {
                     // a new tile's channels
                     ++tile;
                     left = (long long)(rt_hi(tile) - rt_lo(tile)) * n_ks - 1;
                     nch = n_chan(tile);
-                    const int k0 = chan0(tile);
+                    k0 = chan0(tile);
 #pragma unroll
                     for (int i = 0; i < G::ITEMS; ++i) {
                         const int p = pt + i * E_PT, c = p >> 4;
@@ -474,6 +609,9 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                                     : 0.0f;
                     }
                 }
+                if constexpr (RAWX) {
+                    if (gather && !gather_to(it + RAW)) break;
+                }
                 bool ok = mbar_wait(&ctl.raw_full[slot], rph, wc.budget) &&
                           mbar_wait_cluster(&ctl.empty[s], sph ^ 1u, wc.budget);
                 if (!ok) {
@@ -482,9 +620,13 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                 }
                 if (__any_sync(0xffffffffu, !ok || *abort_flag)) break;   // warp-uniform
                 const uint32_t src = ring_u32 + slot * G::RAW_BYTES;
-                chain_rows<KP1, RAWX>(src, v_u32 + s * E_TILE, pt, nch, sc, vf);
+                chain_rows<KP1, RAWX>(src, v_u32 + s * E_TILE, pt, nch, gather,
+                                      (uint32_t)(uintptr_t)W + (uint32_t)k0 * (uint32_t)d * 4u,
+                                      (uint32_t)(uintptr_t)codes + (uint32_t)k0 * (uint32_t)d,
+                                      (uint32_t)d, (uint32_t)C * (uint32_t)d, sc, vf);
                 if constexpr (RAWX)
-                    chain_x<3>(src, x_u32 + s * E_XSET, E_X_EPI + pt, E_ROWS * 16, E_PT, xs);
+                    chain_x<3>(src, x_u32 + s * E_XSET, E_X_EPI + pt, E_ROWS * 16, E_PT, xs, gather,
+                               (uint32_t)(uintptr_t)X, (uint32_t)d);
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl.raw_empty[slot]);
@@ -511,11 +653,17 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                     xph ^= 1u;
                 }
             }
+            if (RAWX && gather) cp_async_wait_all();
         } else if (warp == E_COPY_WARP) {
             // ------------------------------------------------------------ tile copies
             // raw tiles of step f into slot f % RAW once the producers have released step f - RAW,
             // X rows of step f into X slot f % NX once the MMAs of step f - NX have completed
-            if (lane == 0 && wc.withhold == 0) {
+            if (gather && wc.withhold == 0) {
+                if constexpr (RAWX) {
+                    (void)gather_to(total);
+                    cp_async_wait_all();
+                }
+            } else if (lane == 0 && wc.withhold == 0) {
                 prefetch_tensormap(&tmX);
                 prefetch_tensormap(&tmW);
                 prefetch_tensormap(&tmQ);
@@ -670,7 +818,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                 stop = __any_sync(0xffffffffu, !ok || *abort_flag);   // warp-uniform
                 if (stop) break;
                 chain_x<2>(ring_u32 + xslot * G::RAW_BYTES, x_u32 + xstage * E_XSET, et, E_X_EPI,
-                           256, xs);
+                           256, xs, gather, (uint32_t)(uintptr_t)X, (uint32_t)d);
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -860,7 +1008,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
 template <int KP1, bool RAWX>
 mpq_status launch_chain(const float *X, const void *A, int N, const float *W, const int8_t *codes,
                         const float *scales, int C, int d, float *err, const unsigned *xrange,
-                        const unsigned *vrange, void *part, size_t part_bytes,
+                        const unsigned *vrange, const PadRows &pad, void *part, size_t part_bytes,
                         cudaStream_t stream)
 {
     using G = EGeo<KP1, RAWX>;
@@ -871,25 +1019,30 @@ mpq_status launch_chain(const float *X, const void *A, int N, const float *W, co
     memset(&tmX, 0, sizeof(tmX));
     memset(&tmW, 0, sizeof(tmW));
     memset(&tmQ, 0, sizeof(tmQ));
-    bool maps;
+    bool maps = true;
+    const bool gather = RAWX && !tile_rows_ok(X, W, codes, d);   // no tile copies at all
+    const int dp = (d + 15) / 16 * 16;                           // a row of the planes and copies
+    const float *wt = pad.W ? pad.W : W;
+    const int8_t *qt = pad.W ? pad.codes : codes;
     if constexpr (RAWX) {
         const cuuint64_t dx[2] = {(cuuint64_t)d, (cuuint64_t)N}, sx[1] = {(cuuint64_t)d * 4};
         const cuuint32_t bx[2] = {E_KS, E_ROWS};
-        maps = encode_tile_map(&tmX, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, A, dx, sx, bx);
+        if (!gather) maps = encode_tile_map(&tmX, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, A, dx, sx, bx);
     } else {
-        const cuuint64_t dx[3] = {(cuuint64_t)d, (cuuint64_t)N, 2};
-        const cuuint64_t sx[2] = {(cuuint64_t)d * 2, (cuuint64_t)N * d * 2};
+        const cuuint64_t dx[3] = {(cuuint64_t)dp, (cuuint64_t)N, 2};
+        const cuuint64_t sx[2] = {(cuuint64_t)dp * 2, (cuuint64_t)N * dp * 2};
         const cuuint32_t bx[3] = {E_KS, E_ROWS, 2};
         maps = encode_tile_map(&tmX, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, A, dx, sx, bx,
                                CU_TENSOR_MAP_SWIZZLE_128B);
     }
-    const cuuint64_t dw[2] = {(cuuint64_t)d, (cuuint64_t)C}, sw[1] = {(cuuint64_t)d * 4};
+    const cuuint64_t dw[2] = {(cuuint64_t)dp, (cuuint64_t)C}, sw[1] = {(cuuint64_t)dp * 4};
     const cuuint32_t bw[2] = {E_KS, (cuuint32_t)G::CH};
-    const cuuint64_t dq[3] = {(cuuint64_t)d, (cuuint64_t)C, (cuuint64_t)G::K};
-    const cuuint64_t sq[2] = {(cuuint64_t)d, (cuuint64_t)C * d};
+    const cuuint64_t dq[3] = {(cuuint64_t)dp, (cuuint64_t)C, (cuuint64_t)G::K};
+    const cuuint64_t sq[2] = {(cuuint64_t)dp, (cuuint64_t)C * dp};
     const cuuint32_t bq[3] = {E_KS, (cuuint32_t)G::CH, (cuuint32_t)G::K};
-    maps = maps && encode_tile_map(&tmW, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, W, dw, sw, bw) &&
-           encode_tile_map(&tmQ, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, codes, dq, sq, bq);
+    if (!gather)
+        maps = maps && encode_tile_map(&tmW, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, wt, dw, sw, bw) &&
+               encode_tile_map(&tmQ, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, qt, dq, sq, bq);
     if (!maps) {
         set_error("output error: tensor map encoding failed");
         return MPQ_ERR_CUDA;
@@ -985,16 +1138,16 @@ int chain_max_gang(int N) { return N <= E_M ? 1 : E_MAX_GANG; }
 mpq_status launch_output_error_chain(const float *X, int N, const float *W, const int8_t *codes,
                                      const float *scales, int C, int d, int k_max, float *err,
                                      const unsigned *xrange, const unsigned *vrange,
-                                     const uint16_t *xs, void *part, size_t part_bytes,
-                                     cudaStream_t stream)
+                                     const uint16_t *xs, const PadRows &pad, void *part,
+                                     size_t part_bytes, cudaStream_t stream)
 {
     switch (k_max) {
 #define MPQ_CASE(n)                                                                               \
     case n:                                                                                       \
         return xs ? launch_chain<n + 1, false>(X, xs, N, W, codes, scales, C, d, err, xrange,     \
-                                               vrange, part, part_bytes, stream)                  \
+                                               vrange, pad, part, part_bytes, stream)             \
                   : launch_chain<n + 1, true>(X, X, N, W, codes, scales, C, d, err, xrange,       \
-                                              vrange, part, part_bytes, stream);
+                                              vrange, pad, part, part_bytes, stream);
         MPQ_CASE(1) MPQ_CASE(2) MPQ_CASE(3) MPQ_CASE(4) MPQ_CASE(5) MPQ_CASE(6) MPQ_CASE(7)
         MPQ_CASE(8) MPQ_CASE(9) MPQ_CASE(10) MPQ_CASE(11) MPQ_CASE(12) MPQ_CASE(13) MPQ_CASE(14)
         MPQ_CASE(15) MPQ_CASE(16)

@@ -393,6 +393,42 @@ f16_split_kernel(const float4 *__restrict__ X, long long n8, const unsigned *__r
     }
 }
 
+// The same for rows of any length and alignment, into rows of dp elements (zeros from d on).
+__global__ void __launch_bounds__(256)
+f16_split_rows_kernel(const float *__restrict__ X, int N, int d, int dp,
+                      const unsigned *__restrict__ xrange, uint4 *__restrict__ hi,
+                      uint4 *__restrict__ lo)
+{
+    const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
+    const int d8 = dp / 8;
+    const long long n8 = (long long)N * d8, stride = (long long)gridDim.x * blockDim.x;
+    const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long dt = stride / d8;               // rows and items that a stride advances
+    const int dj = (int)(stride - dt * d8);
+    long long t = i0 / d8;
+    int j = (int)(i0 - t * d8);
+    for (long long i = i0; i < n8; i += stride) {
+        const float *x = X + t * d + 8 * j;
+        const int left = d - 8 * j;
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = e < left ? __fmul_rn(__ldg(x + e), xs) : 0.0f;
+        uint4 H, L;
+        split_f16x2(v[0], v[1], H.x, L.x);
+        split_f16x2(v[2], v[3], H.y, L.y);
+        split_f16x2(v[4], v[5], H.z, L.z);
+        split_f16x2(v[6], v[7], H.w, L.w);
+        hi[i] = H;
+        lo[i] = L;
+        t += dt;
+        j += dj;
+        if (j >= d8) {
+            j -= d8;
+            ++t;
+        }
+    }
+}
+
 // Clipping search (Eq. 12): the residual r = w - s q of channel c0 + v / n_cand under candidate
 // v mod n_cand (s = K / Qmax, the codes q of Eq. 8 with the sign of w, q = 0 where s is 0 or NaN),
 // scaled by 2^e and split into fp16 hi/lo planes ([2][M][d] as hi and lo).  One CTA per vector v,
@@ -523,12 +559,19 @@ mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
 
 }  // namespace
 
-// X split into the fp16 planes xs ([2][N][d]) on `stream`.
+// X split into the fp16 planes xs ([2][N][dp]) on `stream`.
 cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange, uint16_t *xs,
                            cudaStream_t stream)
 {
-    const long long n8 = (long long)N * d / 8;
+    const int dp = (d + 15) / 16 * 16;
+    const long long n8 = (long long)N * dp / 8;
     const int sb = (int)std::min<long long>((n8 + 255) / 256, 4LL * sm_count());
+    if (d != dp || ((uintptr_t)X & 15) != 0) {
+        f16_split_rows_kernel<<<(unsigned)std::max(sb, 1), 256, 0, stream>>>(
+            X, N, d, dp, xrange, reinterpret_cast<uint4 *>(xs),
+            reinterpret_cast<uint4 *>(xs + (size_t)N * dp));
+        return cudaGetLastError();
+    }
     f16_split_kernel<<<(unsigned)std::max(sb, 1), 256, 0, stream>>>(
         reinterpret_cast<const float4 *>(X), n8, xrange, reinterpret_cast<uint4 *>(xs),
         reinterpret_cast<uint4 *>(xs + (size_t)N * d));

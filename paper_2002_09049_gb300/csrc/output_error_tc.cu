@@ -1,7 +1,9 @@
 // Output error (Sec. 3.3, Eq. 11) on the 5th-generation tensor cores, single-CTA form:
 //   err[k][n] = (1/N) sum_t (x_t . r_{k,n+1})^2,  n = 0..k_max.
-// It serves the shapes the CTA-pair kernel's TMA tile copies cannot address (rows whose byte
-// length is not a multiple of 16, or unaligned buffers); producers read global memory directly.
+// It serves rows that the CTA-pair kernel's TMA tile copies cannot address (d not a multiple of 16,
+// or unaligned buffers) and for which gathered or copied rows do not pay (short ones, few channels:
+// output_error_rows_ok), and calls whose scratch the pool has no room for; it needs no scratch, and
+// producers read global memory directly.
 //
 // As a contraction: Y = R X^T with R the C*(k_max+1) residual vectors (rows) and X the N
 // calibration rows, both of length d; err is the row-wise mean of Y^2.  Mapping:

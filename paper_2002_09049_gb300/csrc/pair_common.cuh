@@ -49,23 +49,39 @@ bool encode_tile_map(CUtensorMap *m, CUtensorMapDataType type, int rank, const v
                      const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box,
                      CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE);
 
-// Host: max|X| (float bits) into range[0], zeroed first (N d a multiple of 4, X 16-byte aligned).
+// Copies of W and the codes with rows of dp elements, a multiple of 16 (W NULL: none).
+struct PadRows {
+    float *W;        // [C][dp]
+    int8_t *codes;   // [k_max][C][dp]
+    int dp;
+};
+
+// Rows that a tile copy can address: whole multiples of 16 bytes in every array, aligned bases.
+__host__ __device__ inline bool tile_rows_ok(const float *X, const float *W, const int8_t *codes,
+                                             int d)
+{
+    return (d & 15) == 0 && (((uintptr_t)X | (uintptr_t)W | (uintptr_t)codes) & 15) == 0;
+}
+
+// Host: max|X| (float bits) into range[0], zeroed first.
 mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, cudaStream_t stream);
 
-// Host: X * 2^e (e from xrange[0]) split into the fp16 hi and lo planes xs ([2][N][d]).
+// Host: X * 2^e (e from xrange[0]) split into the fp16 hi and lo planes xs ([2][N][dp], dp = d
+// rounded up to 16, the rest of a row zero).
 cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange, uint16_t *xs,
                            cudaStream_t stream);
 
 // Host: the output error of the greedy points (output_error_chain.cu), with its ranges ready on
 // `stream` (xrange[0] = max|X|, vrange = max|r| per residual vector, float bits); xs: the split X
-// planes, or NULL (the contraction then splits X itself); part: part_bytes of 256-byte aligned
+// planes, or NULL (the contraction then splits X itself); pad: padded copies of W and the codes,
+// or none (with xs, W and codes are then rows a tile copy can address); part: part_bytes of 256-byte aligned
 // scratch for partial sums, at least chain_count_bytes(tiles) and that much of it zeroed on
 // `stream` (chain_scratch_bytes(tiles, chain_max_gang(N)) is all it can use).
 mpq_status launch_output_error_chain(const float *X, int N, const float *W, const int8_t *codes,
                                      const float *scales, int C, int d, int k_max, float *err,
                                      const unsigned *xrange, const unsigned *vrange,
-                                     const uint16_t *xs, void *part, size_t part_bytes,
-                                     cudaStream_t stream);
+                                     const uint16_t *xs, const PadRows &pad, void *part,
+                                     size_t part_bytes, cudaStream_t stream);
 int chain_tiles(int C, int k_max);   // channel tiles of a CTA pair
 size_t chain_count_bytes(int tiles);
 size_t chain_scratch_bytes(int tiles, int gang);

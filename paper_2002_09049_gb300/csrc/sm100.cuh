@@ -347,6 +347,32 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
 
 // ---- TMA (bulk tensor copies global -> shared, completion counted on an mbarrier) ------------
 // Arms `bar` for `bytes` of incoming transactions and arrives once.
+// 4 or 16 bytes from global to shared memory, asynchronously; only the first `bytes` are read, the
+// rest is zero.  cp_async_arrive: this thread's arrival on `bar` (in its count) once its copies so
+// far have landed.
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 :: "r"(dst), "l"(__cvta_generic_to_global(src)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 :: "r"(dst), "l"(__cvta_generic_to_global(src)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];"
+                 :: "r"(smem_u32(bar)) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_wait_all()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),

@@ -176,3 +176,36 @@ def test_codes_that_are_not_nearest_values(gpu, oracle, K):
     scales[7] = 1e30                                   # a scale far above its residual, codes 0
     X = wlm.random_calibration(N, d, 5)
     compare_err(gpu_err(X, W, codes, scales, K), oracle.output_error(X, 1, W, codes, scales, K))
+
+
+# rows that tile copies cannot address: around 16 elements and a 64-element step, channel and row
+# tile edges as above, where the chain takes them and just below; off: elements that X, W and
+# (x 4) the codes start past a 16-byte boundary
+@pytest.mark.parametrize("C,d,N,K,off", [(24, 255, 256, 9, 0), (25, 257, 257, 9, 0), (52, 193, 129, 3, 0),
+                                         (51, 193, 300, 3, 0), (52, 191, 300, 3, 0),
+                                         (86, 321, 513, 1, 0), (33, 1039, 1500, 6, 0),
+                                         (15, 601, 300, 16, 0), (700, 207, 700, 4, 0),
+                                         (2000, 300, 128, 8, 0), (43, 256, 300, 4, 1),
+                                         (61, 275, 300, 3, 3)])
+def test_rows_of_any_length(gpu, oracle, C, d, N, K, off):
+    """Padded copies (pooled scratch, with and without the search's ranges) and the gather (fixed
+    scratch) give bit for bit the same errors, within 1e-5 of the oracle."""
+    W = wlm.random_weights(C, d, C + d + K, "t")
+    X = wlm.random_calibration(N, d, 9 + d)
+
+    def t(a, pad):
+        a = torch.from_numpy(np.ascontiguousarray(a)).to(gpu)
+        store = torch.empty(a.numel() + 64, dtype=a.dtype, device=gpu)
+        out = store[pad:pad + a.numel()].view(a.shape)
+        return out.copy_(a)
+
+    o = oracle.quantize_layer(W, 4, 32, K)
+    rmax = np.concatenate([np.abs(W).max(axis=1, keepdims=True),
+                           np.abs(o["residuals"]).max(axis=2).T], axis=1).astype(np.float32)
+    args = (t(X, off), t(W, off), t(o["codes"], 4 * off), t(o["scales"], 0), K)
+    e = binding.mpq_output_error(*args)
+    e_rmax = binding.mpq_output_error(*args, rmax=t(rmax, 0))
+    e_fixed = binding.mpq_output_error_noalloc(*args)
+    torch.cuda.synchronize()
+    assert torch.equal(e, e_fixed) and torch.equal(e, e_rmax)
+    compare_err(e.cpu().numpy(), oracle.output_error(X, 1, W, o["codes"], o["scales"], K))
