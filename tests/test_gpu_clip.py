@@ -31,13 +31,36 @@ def run_both(oracle, X, W, bits, n_cand, mode, groups=1):
     # d % 16 == 0: CTA-pair tensor-core path -- several pair tiles, a part-filled odd CTA, ragged
     # row tiles split over clusters, 1 to 32 candidates
     (50, 256, 600, 20), (13, 64, 100, 32), (130, 128, 300, 7), (3, 48, 20, 1), (64, 576, 512, 20),
-    # other rows: shared-memory path
+    # other rows: fp32 register tiles
     (11, 147, 129, 20), (4, 33, 70, 5), (2, 17, 300, 32),
 ])
 def test_shared_input(gpu, oracle, mode, C, d, N, n_cand):
     W = wlm.random_weights(C, d, 100 + C + d, "laplace")
     X = wlm.random_calibration(N, d, 200 + N)
     run_both(oracle, X, W, 4, n_cand, mode)
+
+
+# tiles of 64 vectors by 128 rows and chunks of 16 elements: one less, exactly and one more of each;
+# row tiles shared by a cluster; off: elements that X and W start past a 16-byte boundary
+@pytest.mark.parametrize("C,d,N,n_cand,off", [(8, 15, 127, 8, 0), (3, 17, 129, 21, 0),
+                                              (13, 31, 128, 5, 0), (1, 1, 1, 1, 0),
+                                              (7, 147, 1025, 32, 0), (2, 33, 5000, 20, 0),
+                                              (300, 75, 260, 20, 0), (5, 64, 300, 20, 1),
+                                              (5, 50, 300, 3, 3)])
+def test_rows_of_any_length(gpu, oracle, C, d, N, n_cand, off):
+    W = wlm.random_weights(C, d, C + d + N, "laplace")
+    X = wlm.random_calibration(N, d, 7 + N)
+
+    def t(a):
+        store = torch.empty(a.size + 8, dtype=torch.float32, device=gpu)
+        return store[off:off + a.size].view(a.shape).copy_(torch.from_numpy(a))
+
+    clip, err, best = binding.mpq_clip_search(t(X), t(W), 4, n_cand)
+    torch.cuda.synchronize()
+    clip, err, best = clip.cpu().numpy(), err.cpu().numpy(), best.cpu().numpy()
+    assert np.array_equal(clip, oracle.clip_candidates(W, n_cand, MODES[0]), equal_nan=True)
+    compare_err(err, oracle.clip_errors(X, 1, W, 4, clip, threads=8))
+    assert np.array_equal(best, oracle.clip_select(err, MODES[0]))
 
 
 @pytest.mark.parametrize("mode", MODES)
