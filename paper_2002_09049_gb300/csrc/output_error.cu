@@ -10,7 +10,10 @@
 // shared memory with coalesced reads (each read once), threads over the rows.
 #include <math.h>
 
+#include <algorithm>
+
 #include "mpq_internal.cuh"
+#include "sm100.cuh"
 
 MPQ_CHECKED_UNIT("output_error.cu");
 
@@ -18,6 +21,143 @@ namespace mpq {
 namespace {
 
 constexpr int GR_THREADS = 256;
+
+// Short rows (every depthwise kernel in use: 9, 25, 49): two rows a thread, so that the k_max+1
+// residuals of an element, read as 16-byte words, serve both, and chunks of X copied with
+// cp.async into one of two buffers while the other is used.  Bound by the latency of the first
+// chunk, then by X's bytes: 960 x 9, k_max = 8, N = 1024 13.0 us (35 MB: 5 us), 1536 x 25 45 us
+// (157 MB: 23 us); the kernel below, one row a thread and a residual per load, is bound by its
+// shared-memory reads: 19.4 and 85 us.
+constexpr int SR_THREADS = 128, SR_ROWS = 2;
+// longer rows come with too few CTAs an SM (two chunks of 256 rows each: 49 elements 23 us either
+// way at 512 channels, N = 512, k_max = 4), and even ones with bank conflicts for both rows
+constexpr int SR_MAX_D = 32;
+constexpr int SR_CHUNK = SR_ROWS * SR_THREADS;    // rows of a chunk
+
+template <int KP1>
+__global__ void __launch_bounds__(SR_THREADS, KP1 <= 9 ? 7 : 4)
+output_error_short_rows_kernel(const float *__restrict__ X, int N, const float *__restrict__ W,
+                               const int8_t *__restrict__ codes, const float *__restrict__ scales,
+                               int C, int d, float *__restrict__ err)
+{
+    constexpr int K = KP1 - 1, KP = (KP1 + 3) / 4 * 4;
+    constexpr int chunk = SR_CHUNK;
+    extern __shared__ __align__(16) float xs[];       // two buffers of chunk * d + 4 floats
+    __shared__ __align__(16) float rsh[SR_MAX_D][KP];
+    __shared__ float red[SR_THREADS / 32][KP1];
+    const int k = blockIdx.x, tid = threadIdx.x;
+    const int buffer = chunk * d + 4;
+    if (!MPQ_IN(k, C) || !MPQ_CHECK(d <= SR_MAX_D) || !MPQ_CHECK_SMEM_END(8 * (size_t)buffer)) return;
+    const uintptr_t x0 = (uintptr_t)X, xk = x0 + (size_t)k * N * d * 4;
+    const int n_chunks = (N + chunk - 1) / chunk;
+    // chunk c into buffer c & 1: the aligned 16 bytes that hold it (none read beyond its end or,
+    // where X itself starts off a boundary, before X)
+    auto copy = [&](int c) {
+        const uintptr_t at = xk + (size_t)c * chunk * d * 4;
+        const int nr = min(chunk, N - c * chunk), off = (int)(at & 15);
+        const int bytes = off + nr * d * 4;
+        const uint32_t dst = sm100::smem_u32(xs + (c & 1) * buffer);
+        const uintptr_t from = at - (unsigned)off;
+        for (int b = 16 * tid; b < bytes; b += 16 * SR_THREADS) {
+            if (from + (unsigned)b < x0) {
+                for (int o = off; o < min(16, bytes); o += 4)
+                    sm100::cp_async4(dst + b + o, reinterpret_cast<const void *>(from + b + o), 4u);
+            } else {
+                sm100::cp_async16(dst + b, reinterpret_cast<const void *>(from + b),
+                                  (uint32_t)min(16, bytes - b));
+            }
+        }
+        sm100::cp_async_commit();
+    };
+    copy(0);
+    if (n_chunks > 1) copy(1);
+
+    for (int j = tid; j < d; j += SR_THREADS) {
+        const size_t at = (size_t)k * d + j, plane = (size_t)C * d;
+        float q[K];
+#pragma unroll
+        for (int n = 0; n < K; ++n) q[n] = (float)__ldg(codes + n * plane + at);
+        float r = __ldg(W + at);
+        rsh[j][0] = r;
+#pragma unroll
+        for (int n = 0; n < K; ++n) {
+            r = __fmaf_rn(-__ldg(scales + (size_t)k * K + n), q[n], r);
+            rsh[j][n + 1] = r;
+        }
+#pragma unroll
+        for (int n = KP1; n < KP; ++n) rsh[j][n] = 0.0f;
+    }
+
+    // squares as in the kernel below: a thread's rows compensated, then a tree over the threads
+    float acc[KP1], comp[KP1];
+#pragma unroll
+    for (int n = 0; n < KP1; ++n) {
+        acc[n] = 0.0f;
+        comp[n] = 0.0f;
+    }
+    for (int c = 0; c < n_chunks; ++c) {
+        if (c + 1 < n_chunks)
+            sm100::cp_async_wait<1>();
+        else
+            sm100::cp_async_wait<0>();
+        __syncthreads();   // this chunk (and the residuals) from every thread
+        const int nr = min(chunk, N - c * chunk);
+        const float *xc = xs + (c & 1) * buffer + ((xk + (size_t)c * chunk * d * 4) & 15) / 4;
+        for (int t = tid; t < nr; t += SR_ROWS * SR_THREADS) {
+            const bool two = t + SR_THREADS < nr;
+            const float *xa = xc + t * d, *xb = two ? xa + SR_THREADS * d : xa;
+            float y[KP], z[KP];
+#pragma unroll
+            for (int n = 0; n < KP; ++n) {
+                y[n] = 0.0f;
+                z[n] = 0.0f;
+            }
+#pragma unroll 3
+            for (int j = 0; j < d; ++j) {
+                const float a = xa[j], b = xb[j];
+#pragma unroll
+                for (int n = 0; n < KP; n += 4) {
+                    const float4 r = *reinterpret_cast<const float4 *>(&rsh[j][n]);
+                    y[n] = fmaf(a, r.x, y[n]);
+                    z[n] = fmaf(b, r.x, z[n]);
+                    if (n + 1 < KP1) {
+                        y[n + 1] = fmaf(a, r.y, y[n + 1]);
+                        z[n + 1] = fmaf(b, r.y, z[n + 1]);
+                    }
+                    if (n + 2 < KP1) {
+                        y[n + 2] = fmaf(a, r.z, y[n + 2]);
+                        z[n + 2] = fmaf(b, r.z, z[n + 2]);
+                    }
+                    if (n + 3 < KP1) {
+                        y[n + 3] = fmaf(a, r.w, y[n + 3]);
+                        z[n + 3] = fmaf(b, r.w, z[n + 3]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < KP1; ++n) {
+                const float p = __fmul_rn(y[n], y[n]);
+                kahan_add(acc[n], comp[n], two ? fmaf(z[n], z[n], p) : p);
+            }
+        }
+        if (c + 2 < n_chunks) {
+            __syncthreads();   // this buffer is no longer read
+            copy(c + 2);
+        }
+    }
+    const int lane = tid & 31, wp = tid >> 5;
+#pragma unroll
+    for (int n = 0; n < KP1; ++n) {
+        kahan_add(acc[n], comp[n], 0.0f);
+        float v = acc[n];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[wp][n] = v;
+    }
+    __syncthreads();
+    if (tid < KP1 && MPQ_IN((size_t)k * KP1 + tid, (size_t)C * KP1))
+        err[(size_t)k * KP1 + tid] =
+            mean_of_sum((red[0][tid] + red[2][tid]) + (red[1][tid] + red[3][tid]), N);
+}
 
 constexpr int GR_X_FLOATS = 4096;                 // 16 KB of calibration rows staged at a time
 
@@ -115,6 +255,16 @@ template <int KP1>
 mpq_status launch_grouped(const float *X, int N, const float *W, const int8_t *codes,
                           const float *scales, int C, int d, float *err, cudaStream_t stream)
 {
+    if (d <= SR_MAX_D) {
+        const int bytes = 2 * (SR_CHUNK * d + 4) * (int)sizeof(float);   // 66 KB at most
+        static std::atomic<int> limit[kMaxDevices];
+        const cudaError_t e = allow_smem(
+            reinterpret_cast<const void *>(output_error_short_rows_kernel<KP1>), limit, bytes);
+        if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
+        output_error_short_rows_kernel<KP1><<<C, SR_THREADS, bytes, stream>>>(X, N, W, codes, scales, C,
+                                                                             d, err);
+        return cuda_status(cudaGetLastError(), "grouped output-error kernel launch");
+    }
     const size_t smem = ((size_t)(KP1 * d + 3) / 4 * 4 + GR_X_FLOATS) * sizeof(float);
     if (d > GR_X_FLOATS || (long long)smem > max_smem_optin()) {
         set_error("groups = C with d = %d and k_max = %d needs %zu bytes of shared memory", d,

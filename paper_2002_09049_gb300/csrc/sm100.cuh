@@ -368,6 +368,18 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *bar)
                  :: "r"(smem_u32(bar)) : "memory");
 }
 
+__device__ __forceinline__ void cp_async_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// This thread's groups but the newest `n` have landed.
+template <int n>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" :: "n"(n) : "memory");
+}
+
 __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.wait_all;" ::: "memory");

@@ -38,7 +38,10 @@ def test_shared_input(gpu, oracle, C, d, N, K):
 
 
 @pytest.mark.parametrize("C,d,N,K", [(1, 9, 1, 1), (6, 9, 100, 8), (40, 9, 1024, 8), (3, 25, 77, 4),
-                                     (5, 300, 33, 16)])
+                                     (5, 300, 33, 16),
+                                     # two rows a thread: chunks of 256 rows, 32 elements at most
+                                     (3, 32, 257, 8), (3, 33, 257, 8), (7, 9, 255, 3), (2, 31, 513, 16),
+                                     (4, 1, 1025, 1), (5, 16, 129, 9)])
 def test_per_channel_input(gpu, oracle, C, d, N, K):
     W = wlm.random_weights(C, d, 3 * C + d, "laplace")
     q = oracle.quantize_layer(W, 4, 64, K)
