@@ -309,8 +309,8 @@ mpq_status mpq_center_weights(const float *W, int C, int d, int mode, float *cen
  * Scratch: with groups == 1, d a multiple of 16 and X, W 16-byte aligned (the tensor-core path),
  * 4 C + 4 N d bytes (channel maxima, X's fp16 hi/lo planes) and the fp16 hi/lo planes of the
  * candidates' residuals, 4 d n_cand bytes per channel for at most max(1, 2^32 / (4 d n_cand))
- * channels at a time (larger layers run in chunks of whole channels), come from the current
- * device's stream-ordered pool on `stream` in one allocation (as for mpq_output_error;
+ * channels at a time (larger layers run in chunks of whole channels), and about 5 MB at most of
+ * partial sums (with 8 bytes per 256 residual vectors), come from the current device's stream-ordered pool on `stream` in one allocation (as for mpq_output_error;
  * MPQ_ERR_NOMEM if it has no room, and nothing else is enqueued then).
  */
 mpq_status mpq_clip_search(const float *X, int N, int groups, const float *W, int C, int d,

@@ -13,6 +13,12 @@
 //   memory ([2][N][d]), and clip_planes_kernel writes every candidate's residual as such planes;
 //   tile copies put each 64-element step straight into the operand tiles (128-byte swizzle).
 // * Work advances in steps of 64 elements (one 128-byte row of fp16 per operand row).
+// * Resident pairs take units (vector tile, part of its row tiles) in turn, so that pairs at work at
+//   the same time share vector tiles (from L2) and none has more than one unit above the mean
+//   (20000 vectors, N = 2048: 9 row tiles on the busiest pair; whole vector tiles to clusters of four
+//   pairs: 10; 1000 x 2048, N = 2048, 20 candidates 424 -> 343 us with one commit a step for both
+//   operands).  A vector tile's parts are summed through global scratch, by the last to
+//   arrive, in order.
 // * Two accumulators in tensor memory (columns [0, 256) and [256, 512)) take alternate segments,
 //   and the running sums live in the epilogue warps' registers (one TMEM lane x 128 columns per
 //   thread; setmaxnreg moves registers from warpgroups 0-1 to the epilogue's), so the MMA thread
@@ -49,8 +55,7 @@ constexpr int F_VEC = 128;                 // residual vectors per CTA (TMEM lan
 constexpr int F_ROWS = 128;                // calibration rows per CTA
 constexpr int F_N = 2 * F_ROWS;            // rows per pair row tile (UMMA N)
 constexpr int F_KS = 64;                   // elements per step: one 128-byte fp16 row
-constexpr int F_ASETS = 3;                 // A operand stages (tile sets)
-constexpr int F_BSLOTS = 3;                // B operand slots
+constexpr int F_STAGES = 3;                // operand stages (an A and a B tile set each)
 constexpr int F_SEG = 4;                   // steps per accumulation segment (256 elements)
 constexpr int F_MMA_WARP = 7;              // MMA issuer
 constexpr int F_EPI_WARP0 = 8;             // a multiple of 4: warp % 4 is the TMEM lane quarter
@@ -68,69 +73,70 @@ constexpr uint32_t F_TMEM_COLS = 512;
 constexpr int F_SMEM_LIMIT = 232448;       // opt-in shared memory per CTA on sm_100 parts
 
 struct F16Ctrl {
-    uint64_t full[F_ASETS];    // even CTA: both CTAs' relays (A and B landed)
-    uint64_t empty[F_ASETS];   // both CTAs: pair MMA commit (A stage free)
-    uint64_t afull[F_ASETS];   // this CTA's A tile copy
-    uint64_t bfull[F_BSLOTS];      // this CTA's B tile copy
-    uint64_t bempty[F_BSLOTS];     // both CTAs: pair MMA commit (B slot free)
-    uint64_t segfull[2];           // both CTAs: pair MMA commit, per accumulator
-    uint64_t segempty[2];          // even CTA: both CTAs' epilogue warps, per accumulator
-    uint64_t done;                 // even CTA: every MMA complete
+    uint64_t full[F_STAGES];   // even CTA: both CTAs' relays (A and B landed)
+    uint64_t empty[F_STAGES];  // both CTAs: pair MMA commit (stage free)
+    uint64_t landed[F_STAGES]; // this CTA's A and B tile copies
+    uint64_t segfull[2];       // both CTAs: pair MMA commit, per accumulator
+    uint64_t segempty[2];      // even CTA: both CTAs' epilogue warps, per accumulator
+    uint64_t done;             // even CTA: every MMA complete
     uint32_t tmem_base;
     int abort;
-    double part[2][F_VEC];         // per column half: sum over the rows' y^2
-    int vexp[F_VEC];               // e of every residual vector
+    int last[2];               // this CTA was the last to leave a tile's sums (alternate units)
+    double part[2][F_VEC];     // the upper column half's sums over y^2 (alternate units)
     int xexp;
 };
 constexpr int F_CTRL_BYTES = (sizeof(F16Ctrl) + 1023) / 1024 * 1024;
-constexpr int F_SMEM = 1024 + F_CTRL_BYTES + (F_ASETS + F_BSLOTS) * F_SET;
+constexpr int F_SMEM = 1024 + F_CTRL_BYTES + F_STAGES * 2 * F_SET;
 static_assert(F_SMEM <= F_SMEM_LIMIT, "clipping search: shared memory");
+
+// Partial sums of a vector tile's parts, in global scratch, by tile and CTA of the pair: how many
+// have arrived (zeroed before the launch), and 2 F_VEC sums per part.
+struct ClipScratch {
+    unsigned *count;   // [tiles][2]
+    double *slot;      // [tiles][parts][2][F_VEC]
+};
 
 // C residual vectors, given as fp16 hi/lo planes (tmA: [2][C][d], clip_planes_kernel); vrange: the
 // bound on each vector's elements that set its operand scale; xrange[0]: max|X|, both as float
-// bits; tmX: the split X planes [2][N][d] fp16.
+// bits; tmX: the split X planes [2][N][d] fp16.  parts: of a vector tile's row tiles, each one unit.
 __global__ void __launch_bounds__(F_THREADS, 1)
 clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
-                  const unsigned *__restrict__ vrange, float *__restrict__ err, int split,
-                  const WaitCtl wc, const __grid_constant__ CUtensorMap tmX,
+                  const unsigned *__restrict__ vrange, float *__restrict__ err, int parts,
+                  const ClipScratch scratch, const WaitCtl wc,
+                  const __grid_constant__ CUtensorMap tmX,
                   const __grid_constant__ CUtensorMap tmA)
 {
-    constexpr int NA = F_ASETS, NB = F_BSLOTS, SEG = F_SEG;
+    constexpr int NS = F_STAGES, SEG = F_SEG;
     constexpr unsigned KBIT = MPQ_TIMEOUT_CLIP;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw_u32 = smem_u32(smem_raw);
     const uint32_t pad = (1024u - (raw_u32 & 1023u)) & 1023u;
     F16Ctrl &ctl = *reinterpret_cast<F16Ctrl *>(smem_raw + pad);
-    const uint32_t a_u32 = raw_u32 + pad + F_CTRL_BYTES;
-    const uint32_t b_u32 = a_u32 + NA * F_SET;
+    const uint32_t a_u32 = raw_u32 + pad + F_CTRL_BYTES;   // stages of an A and a B set
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t crank = cluster_ctarank();
-    const int half = (int)(crank & 1u);              // 0: even CTA (issues the MMAs), 1: its peer
-    const uint32_t leader = crank & ~1u;
-    const uint16_t pair_mask = (uint16_t)(3u << leader);
-    const int pr = (int)(crank >> 1);                // pair index in the cluster: row-tile phase
-    const int pair_tile = blockIdx.x / (2 * split);
-    const int k0 = (pair_tile * 2 + half) * F_VEC;   // first vector of this CTA
-    const int nvec = max(0, min(F_VEC, C - k0));
+    const int half = (int)cluster_ctarank();         // 0: even CTA (issues the MMAs), 1: its peer
+    const uint16_t pair_mask = 3u;
     const int n_rt = (N + F_N - 1) / F_N;
-    const int my_rt = (n_rt - pr + split - 1) / split;
     const int n_ks = (d + F_KS - 1) / F_KS;          // steps per row tile
     const int nseg = (n_ks + SEG - 1) / SEG;
-    const int total = my_rt * n_ks;
+    // this pair's units: every n_pairs-th of (vector tile, part of its row tiles)
+    const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
+    const int units = (C + 2 * F_VEC - 1) / (2 * F_VEC) * parts;
+    auto vec0 = [&](int u) { return (u / parts * 2 + half) * F_VEC; };   // this CTA's first vector
+    auto rt_lo = [&](int u) { return (int)((long long)n_rt * (u % parts) / parts); };
+    auto rt_hi = [&](int u) { return (int)((long long)n_rt * (u % parts + 1) / parts); };
+    long long total = 0;                             // steps
+    for (int u = pair; u < units; u += n_pairs) total += (long long)(rt_hi(u) - rt_lo(u)) * n_ks;
     // control block and operand tiles within the launch's shared memory (the same in every CTA, so
     // the whole cluster leaves together)
-    if (!MPQ_CHECK_SMEM_END((size_t)pad + F_CTRL_BYTES + (size_t)(NA + NB) * F_SET)) return;
+    if (!MPQ_CHECK_SMEM_END((size_t)pad + F_CTRL_BYTES + (size_t)NS * 2 * F_SET)) return;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NA; ++s) {
+        for (int s = 0; s < NS; ++s) {
             mbar_init(&ctl.full[s], 2);
             mbar_init(&ctl.empty[s], 1);
-            mbar_init(&ctl.afull[s], 1);
-        }
-        for (int s = 0; s < NB; ++s) {
-            mbar_init(&ctl.bfull[s], 1);
-            mbar_init(&ctl.bempty[s], 1);
+            mbar_init(&ctl.landed[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&ctl.segfull[b], 1);
@@ -138,13 +144,9 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
         }
         mbar_init(&ctl.done, 1);
         ctl.abort = 0;
+        ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
         fence_barrier_init();
     }
-    for (int i = threadIdx.x; i < nvec; i += F_THREADS) {
-        if (!MPQ_IN(k0 + i, C)) continue;
-        ctl.vexp[i] = f16_scale_exp(__uint_as_float(__ldg(vrange + k0 + i)));
-    }
-    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
     if (warp == F_MMA_WARP) {
         tmem_alloc_pair(&ctl.tmem_base, F_TMEM_COLS);
         tc_fence_before();
@@ -160,53 +162,48 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
         if (warp == 0) {
             // ------------------------------------------------------------ relay
             // a step's A and B tiles of this CTA have landed: report the stage full
-            int s = 0, sb = 0;
-            uint32_t aph = 0, bph = 0;
-            for (int it = 0; it < total; ++it) {
-                const bool ok = mbar_wait(&ctl.afull[s], aph, wc.budget) &&
-                                mbar_wait(&ctl.bfull[sb], bph, wc.budget);
+            int s = 0;
+            uint32_t ph = 0;
+            for (long long it = 0; it < total; ++it) {
+                const bool ok = mbar_wait(&ctl.landed[s], ph, wc.budget);
                 if (!ok) {
                     *abort_flag = 1;
                     note_timeout(wc, KBIT);
                 }
                 if (__any_sync(0xffffffffu, !ok || *abort_flag)) break;   // warp-uniform
-                if (lane == 0) mbar_arrive_cluster(&ctl.full[s], leader);
-                if (++s == NA) {
+                if (lane == 0) mbar_arrive_cluster(&ctl.full[s], 0);
+                if (++s == NS) {
                     s = 0;
-                    aph ^= 1u;
-                }
-                if (++sb == NB) {
-                    sb = 0;
-                    bph ^= 1u;
+                    ph ^= 1u;
                 }
             }
         } else if (warp == F_MMA_WARP && half == 0 && lane == 0) {
             // ------------------------------------------------------------ MMA issuer (even CTA)
             constexpr uint32_t idesc = idesc_f16(2 * F_VEC, F_N);
             bool ok = true;
-            // step it = (row tile, step ks), stage s, B slot sb, segment g (accumulator g & 1)
-            int ks = 0, s = 0, sb = 0, g = 0, sk = 0;
-            uint32_t aph = 0;
-            for (int it = 0; it < total && ok && !*abort_flag; ++it) {
+            // step it = (row tile, step ks), stage s, segment g (accumulator g & 1)
+            int ks = 0, s = 0, sk = 0;
+            unsigned g = 0;
+            uint32_t ph = 0;
+            for (long long it = 0; it < total && ok && !*abort_flag; ++it) {
                 const bool seg_start = sk == 0;
-                const uint32_t b = (uint32_t)g & 1u;
+                const uint32_t b = g & 1u;
                 if (seg_start) {
                     // this accumulator's previous segment has been folded by both epilogues
-                    if (!mbar_wait_cluster(&ctl.segempty[b], ((uint32_t)(g >> 1) & 1u) ^ 1u,
-                                           wc.budget)) {
+                    if (!mbar_wait_cluster(&ctl.segempty[b], ((g >> 1) & 1u) ^ 1u, wc.budget)) {
                         note_timeout(wc, KBIT);
                         ok = false;
                         break;
                     }
                     tc_fence_after();
                 }
-                if (!mbar_wait_cluster(&ctl.full[s], aph, wc.budget)) {
+                if (!mbar_wait_cluster(&ctl.full[s], ph, wc.budget)) {
                     note_timeout(wc, KBIT);
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t aset = a_u32 + s * F_SET, bset = b_u32 + sb * F_SET;
+                const uint32_t aset = a_u32 + s * 2 * F_SET, bset = aset + F_SET;
                 const uint64_t ah = smem_desc_sw128(aset), al = smem_desc_sw128(aset + F_TILE);
                 const uint64_t bh = smem_desc_sw128(bset), bl = smem_desc_sw128(bset + F_TILE);
                 const uint32_t dt = tmem + b * (F_TMEM_COLS / 2);
@@ -220,7 +217,6 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
                     mma_f16_pair(dt, ah + o, bh + o, idesc, 1u);
                 }
                 mma_commit_pair(&ctl.empty[s], pair_mask);
-                mma_commit_pair(&ctl.bempty[sb], pair_mask);
                 ++ks;
                 if (++sk == SEG || ks == n_ks) {
                     mma_commit_pair(&ctl.segfull[b], pair_mask);
@@ -228,15 +224,14 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
                     ++g;
                 }
                 if (ks == n_ks) ks = 0;
-                if (++s == NA) {
+                if (++s == NS) {
                     s = 0;
-                    aph ^= 1u;
+                    ph ^= 1u;
                 }
-                if (++sb == NB) sb = 0;
             }
             if (!ok) *abort_flag = 1;
             // drain: every MMA issued above completes before tensor memory is released
-            mma_commit_pair(&ctl.done, (uint16_t)(1u << leader));
+            mma_commit_pair(&ctl.done, (uint16_t)1u);
             drain_wait_cluster(&ctl.done, 0, wc, KBIT);
         }
         __syncwarp();
@@ -246,91 +241,93 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
         // lane quarter q (the TMEM lanes this warp may access) and column half h; the running sums
         // of this thread's TMEM lane over the half's 128 columns stay in registers
         const int ew = warp - F_EPI_WARP0, q = ew & 3, h = ew >> 2;
+        const int m = q * 32 + lane;                 // this thread's vector of the CTA's
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * (F_N / 2));
-        const int nseg_all = my_rt * nseg;
         float sums[F_N / 2];
-        double acc = 0.0;
         // Warp F_COPY_WARP also issues the CTA's tile copies, step by step: A and B tiles of step f
-        // once the MMAs of the step that held their slot have completed.  It goes on copying until
+        // once the MMAs of the step that held their stage have completed.  It goes on copying until
         // the next segment has ended, then folds it like the other epilogue warps (a segment ends
         // every SEG steps, and its fold is needed only SEG steps later, when its accumulator is
         // taken again).
         const bool copier = warp == F_COPY_WARP && wc.withhold == 0;
-        int next = 0, a_issued = 0, b_issued = 0;
+        long long next = 0, issued = 0;
+        int cks = 0, cu = pair, crt = rt_lo(pair), cs = 0;   // step, unit, row tile, stage to copy
+        uint32_t cph = 1;
         if (copier && lane == 0) {
             prefetch_tensormap(&tmX);
             prefetch_tensormap(&tmA);
         }
-        for (int g = 0; g < nseg_all; ++g) {
-            const uint32_t b = (uint32_t)g & 1u, par = (uint32_t)(g >> 1) & 1u;
-            bool ok = true;
-            if (copier) {
-                while (next < total) {
-                    if (lane == 0) {
-                        const int f = next, x = (f % n_ks) * F_KS;
-                        const int bslot = f % NB;
-                        const uint32_t bdst = b_u32 + bslot * F_SET;
-                        const int row0 = (pr + (f / n_ks) * split) * F_N + half * F_ROWS;
-                        // a tile copy starts 16-byte aligned (fp16 elements) into a 1024-byte
-                        // aligned destination (128-byte swizzle), or is not issued and the launch
-                        // ends through the bounded waits
-                        const int as = f % NA;
-                        const uint32_t adst = a_u32 + as * F_SET;
-                        ok = MPQ_CHECK((x & 7) == 0 && (adst & 1023u) == 0u &&
-                                       (bdst & 1023u) == 0u && x < d);
-                        if (ok && f >= NA)
-                            ok = mbar_wait_cluster(&ctl.empty[as], (uint32_t)((f - NA) / NA) & 1u,
-                                                   wc.budget);
-                        if (ok) {
-                            mbar_arrive_expect_tx(&ctl.afull[as], 2 * F_TILE);
-                            tma_load_3d(adst, &tmA, x, k0, 0, &ctl.afull[as]);
-                            a_issued = f + 1;
-                        }
-                        if (ok && f >= NB)
-                            ok = mbar_wait_cluster(&ctl.bempty[bslot], (uint32_t)((f - NB) / NB) & 1u,
-                                                   wc.budget);
-                        if (ok) {
-                            mbar_arrive_expect_tx(&ctl.bfull[bslot], 2 * F_TILE);
-                            tma_load_3d(bdst, &tmX, x, row0, 0, &ctl.bfull[bslot]);
-                            b_issued = f + 1;
-                        }
-                    }
-                    ++next;
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) break;
-                    // stop copying once segment g has ended
-                    const bool ended = mbar_test_cluster(&ctl.segfull[b], par);
-                    if (__shfl_sync(0xffffffffu, ended, 0)) break;
-                }
-            }
-            ok = ok && mbar_wait_cluster(&ctl.segfull[b], par, wc.budget);
-            if (!ok) {
-                *abort_flag = 1;
-                note_timeout(wc, KBIT);
-            }
-            if (__any_sync(0xffffffffu, !ok || *abort_flag)) break;   // warp-uniform
-            // fold segment g (accumulator b) into the sums; the last segment of a row tile adds
-            // the rows' y^2 into acc
-            tc_fence_after();
-            const int sg = g % nseg;
-            // a row tile's sums start from zero (0 + v = v, up to the sign of a zero, which the
-            // squares below do not see)
-            if (sg == 0) {
+        unsigned g = 0;             // segment
+        int un = 0;                 // units done
+        bool stop = false;          // given up: no more waits, sums are NaN (warp-uniform)
+        for (int u = pair; u < units; u += n_pairs, ++un) {
+            double acc = 0.0;
+            for (int rt = rt_lo(u); rt < rt_hi(u) && !stop; ++rt) {
+                // a row tile's sums start from zero (0 + v = v, up to the sign of a zero, which the
+                // squares below do not see)
 #pragma unroll
                 for (int i = 0; i < F_N / 2; ++i) sums[i] = 0.0f;
-            }
+                for (int sg = 0; sg < nseg; ++sg, ++g) {
+                    const uint32_t b = g & 1u, par = (g >> 1) & 1u;
+                    bool ok = true;
+                    if (copier) {
+                        while (next < total) {
+                            if (lane == 0) {
+                                const int x = cks * F_KS;
+                                const uint32_t adst = a_u32 + cs * 2 * F_SET;
+                                // a tile copy starts 16-byte aligned (fp16 elements) into a
+                                // 1024-byte aligned destination (128-byte swizzle), or is not
+                                // issued and the launch ends through the bounded waits
+                                ok = MPQ_CHECK((x & 7) == 0 && (adst & 1023u) == 0u && x < d);
+                                if (ok && next >= NS)
+                                    ok = mbar_wait_cluster(&ctl.empty[cs], cph, wc.budget);
+                                if (ok) {
+                                    mbar_arrive_expect_tx(&ctl.landed[cs], 4 * F_TILE);
+                                    tma_load_3d(adst, &tmA, x, vec0(cu), 0, &ctl.landed[cs]);
+                                    tma_load_3d(adst + F_SET, &tmX, x, crt * F_N + half * F_ROWS, 0,
+                                                &ctl.landed[cs]);
+                                    issued = next + 1;
+                                }
+                            }
+                            ++next;
+                            if (++cks == n_ks) {
+                                cks = 0;
+                                if (++crt == rt_hi(cu) && (cu += n_pairs) < units) crt = rt_lo(cu);
+                            }
+                            if (++cs == NS) {
+                                cs = 0;
+                                cph ^= 1u;
+                            }
+                            ok = __shfl_sync(0xffffffffu, ok, 0);
+                            if (!ok) break;
+                            // stop copying once segment g has ended
+                            const bool ended = mbar_test_cluster(&ctl.segfull[b], par);
+                            if (__shfl_sync(0xffffffffu, ended, 0)) break;
+                        }
+                    }
+                    ok = ok && mbar_wait_cluster(&ctl.segfull[b], par, wc.budget);
+                    if (!ok) {
+                        *abort_flag = 1;
+                        note_timeout(wc, KBIT);
+                    }
+                    stop = __any_sync(0xffffffffu, !ok || *abort_flag);
+                    if (stop) break;
+                    // fold segment g (accumulator b) into the sums
+                    tc_fence_after();
 #pragma unroll
-            for (int cb = 0; cb < F_N / 64; ++cb) {
-                float v[32];
-                tmem_ld_32x32b_x32(lane_base + b * (F_TMEM_COLS / 2) + (uint32_t)(cb * 32), v);
+                    for (int cb = 0; cb < F_N / 64; ++cb) {
+                        float v[32];
+                        tmem_ld_32x32b_x32(lane_base + b * (F_TMEM_COLS / 2) + (uint32_t)(cb * 32), v);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) sums[cb * 32 + i] = __fadd_rn(v[i], sums[cb * 32 + i]);
-            }
-            // the accumulator is free again (the loads have completed)
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(&ctl.segempty[b], leader);
-            if (sg == nseg - 1) {
+                        for (int i = 0; i < 32; ++i)
+                            sums[cb * 32 + i] = __fadd_rn(v[i], sums[cb * 32 + i]);
+                    }
+                    // the accumulator is free again (the loads have completed)
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(&ctl.segempty[b], 0);
+                }
+                if (stop) break;
 #pragma unroll
                 for (int cb = 0; cb < F_N / 64; ++cb) {
                     float p = 0.0f;
@@ -339,34 +336,47 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
                     acc += (double)p;
                 }
             }
+            // ---- the end of a unit, reached by every epilogue warp also when it has given up
+            const int ub = un & 1, tile = u / parts;
+            if (h == 1) ctl.part[ub][m] = acc;
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (h == 0) {
+                double s = acc + ctl.part[ub][m];
+                if (*abort_flag) s = (double)NAN;
+                bool write = true;
+                if (parts > 1) {   // this part's sums into scratch; the last one adds them in order
+                    double *slots = scratch.slot + ((size_t)tile * parts * 2 + half) * F_VEC + m;
+                    slots[(size_t)(u - tile * parts) * 2 * F_VEC] = s;
+                    __threadfence();
+                    asm volatile("bar.sync 2, 128;" ::: "memory");
+                    if (m == 0)
+                        ctl.last[ub] = atomicAdd(scratch.count + 2 * (size_t)tile + half, 1u) ==
+                                       (unsigned)(parts - 1);
+                    asm volatile("bar.sync 2, 128;" ::: "memory");
+                    write = ctl.last[ub] != 0;
+                    if (write) {
+                        __threadfence();
+                        s = 0.0;
+                        for (int p = 0; p < parts; ++p) s += __ldcg(slots + (size_t)p * 2 * F_VEC);
+                    }
+                }
+                const int v = vec0(u) + m;
+                if (write && v < C && MPQ_IN(v, C)) {
+                    // exact: undo the operand scales
+                    const int e = ctl.xexp + f16_scale_exp(__uint_as_float(__ldg(vrange + v)));
+                    err[v] = (float)(s / (double)N * pow2d(-2 * e));
+                }
+            }
         }
-        // no copy lands after the CTA is gone: the last copy of every slot
+        // no copy lands after the CTA is gone: the last copy of every stage
         if (copier && lane == 0) {
-            for (int f = a_issued - NA > 0 ? a_issued - NA : 0; f < a_issued; ++f)
-                drain_wait(&ctl.afull[f % NA], (uint32_t)(f / NA) & 1u, wc, KBIT);
-            for (int f = b_issued - NB > 0 ? b_issued - NB : 0; f < b_issued; ++f)
-                drain_wait(&ctl.bfull[f % NB], (uint32_t)(f / NB) & 1u, wc, KBIT);
+            for (long long f = issued - NS > 0 ? issued - NS : 0; f < issued; ++f)
+                drain_wait(&ctl.landed[f % NS], (uint32_t)(f / NS) & 1u, wc, KBIT);
         }
         __syncwarp();
-        ctl.part[h][q * 32 + lane] = *abort_flag ? (double)NAN : acc;
     }
 
-    // ---------------------------------------------------------------- cluster reduction
-    cluster_sync();
-    if (crank < 2 && warp >= F_EPI_WARP0 && warp < F_EPI_WARP0 + 4) {
-        const int m = (warp - F_EPI_WARP0) * 32 + lane;
-        if (m < nvec) {
-            double s = 0.0;
-            for (int j = 0; j < split; ++j) {
-                s += ld_dsmem_f64(&ctl.part[0][m], crank + 2u * (uint32_t)j);
-                s += ld_dsmem_f64(&ctl.part[1][m], crank + 2u * (uint32_t)j);
-            }
-            double v = s / (double)N;
-            v *= pow2d(-2 * (ctl.xexp + ctl.vexp[m]));   // exact: undo the operand scales
-            if (MPQ_IN(k0 + m, C)) err[k0 + m] = (float)v;
-        }
-    }
-    cluster_sync();
+    cluster_sync();   // nothing of the pair's is in flight
     if (warp == F_MMA_WARP) {
         tc_fence_after();
         tmem_dealloc_pair(tmem, F_TMEM_COLS);
@@ -478,13 +488,30 @@ clip_planes_kernel(const float *__restrict__ W, int d, const float *__restrict__
     }
 }
 
-// The contraction over the residual planes A of C vectors, X already split into xs.
+int clip_tiles(int vectors) { return (vectors + 2 * F_VEC - 1) / (2 * F_VEC); }
+
+// Parts of a vector tile's row tiles: single row tiles up to about 16 units a pair, larger parts
+// beyond (the scratch of their sums stays below about 5 MB), never more than row tiles.
+int clip_parts(int tiles, int N)
+{
+    const long long n_rt = (N + (long long)F_N - 1) / F_N;
+    const long long per = std::max(1LL, tiles * n_rt / (16LL * (sm_count() / 2)));
+    return (int)((n_rt + std::min(per, n_rt) - 1) / std::min(per, n_rt));
+}
+
+size_t clip_slot_bytes(int tiles, int N)
+{
+    const int parts = clip_parts(tiles, N);
+    return parts > 1 ? (size_t)tiles * parts * 2 * F_VEC * sizeof(double) : 0;
+}
+
+// The contraction over the residual planes A of C vectors, X already split into xs; count, slot:
+// ClipScratch of clip_tiles(C) tiles.
 mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
                              const unsigned *xrange, const unsigned *vrange, const uint16_t *xs,
-                             cudaStream_t stream)
+                             unsigned *count, double *slot, cudaStream_t stream)
 {
-    const int n_pairs = (C + 2 * F_VEC - 1) / (2 * F_VEC);
-    const int n_rt = (N + F_N - 1) / F_N;
+    const int tiles = clip_tiles(C), parts = clip_parts(tiles, N);
 
     CUtensorMap tmX, tmA;
     memset(&tmX, 0, sizeof(tmX));
@@ -506,8 +533,8 @@ mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
         set_error("clipping search needs %d bytes of shared memory", F_SMEM);
         return MPQ_ERR_UNSUPPORTED;
     }
-    cudaError_t e = cudaFuncSetAttribute(clip_error_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM);
+    static std::atomic<int> limit[kMaxDevices];
+    cudaError_t e = allow_smem(reinterpret_cast<const void *>(clip_error_kernel), limit, F_SMEM);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
 
     cudaLaunchConfig_t cfg = {};
@@ -516,44 +543,29 @@ mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-
-    // Row tiles split over `split` pairs per cluster (clusters of 2 * split CTAs): the split with
-    // the least (waves of resident clusters) x (row tiles per CTA), ties to the larger cluster,
-    // whose pairs read the same A tiles at about the same time (from L2); resident clusters per cluster size queried once per
-    // process (one device per process).
-    static std::atomic<int> resident[3] = {{0}, {0}, {0}};
-    int split = 1;
-    long long best = -1;
-    for (int sp = 1, i = 0; sp <= 4 && sp <= n_rt; sp *= 2, ++i) {
-        attr[0].val.clusterDim.x = (unsigned)(2 * sp);
-        cfg.gridDim = dim3((unsigned)(n_pairs * 2 * sp), 1, 1);
-        int active = resident[i].load(std::memory_order_relaxed);
-        if (active == 0) {
-            if (cudaOccupancyMaxActiveClusters(&active, clip_error_kernel, &cfg) !=
-                cudaSuccess)
-                active = -1;
-            (void)cudaGetLastError();
-            resident[i].store(active, std::memory_order_relaxed);
-        }
-        if (active < 1) continue;
-        const long long waves = (n_pairs + active - 1) / active;
-        const long long cost = waves * ((n_rt + sp - 1) / sp);
-        if (best < 0 || cost <= best) {
-            best = cost;
-            split = sp;
-        }
+    // one resident pair per two SMs (queried once per process), no more than units
+    static std::atomic<int> resident{0};
+    int pairs = resident.load(std::memory_order_relaxed);
+    if (pairs == 0) {
+        cfg.gridDim = dim3((unsigned)(sm_count() / 2 * 2), 1, 1);
+        e = cudaOccupancyMaxActiveClusters(&pairs, clip_error_kernel, &cfg);
+        if (e != cudaSuccess) return cuda_status(e, "cudaOccupancyMaxActiveClusters");
+        pairs = std::max(1, pairs);
+        resident.store(pairs, std::memory_order_relaxed);
     }
-    attr[0].val.clusterDim.x = (unsigned)(2 * split);
-    cfg.gridDim = dim3((unsigned)(n_pairs * 2 * split), 1, 1);
+    pairs = std::min(pairs, tiles * parts);
+    cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
+    const ClipScratch scratch = {count, slot};
     WaitCtl wc;
     mpq_status wst = wait_ctl(&wc);
     if (wst != MPQ_OK) return wst;
-    e = cudaLaunchKernelEx(&cfg, clip_error_kernel, C, N, d, xrange, vrange, err, split, wc, tmX,
-                           tmA);
+    e = cudaLaunchKernelEx(&cfg, clip_error_kernel, C, N, d, xrange, vrange, err, parts, scratch, wc,
+                           tmX, tmA);
     return cuda_status(e, "clipping-search kernel launch");
 }
 
@@ -584,26 +596,50 @@ static int clip_chunk_channels(int C, int d, int n_cand)
     return (int)std::min<long long>(C, std::max(1LL, (1LL << 32) / (4LL * d * n_cand)));
 }
 
+// The X range word, X's planes, the residual planes of one chunk, their bounds, the partial sums of
+// one chunk, the arrival counters of every chunk.
+struct ClipLayout {
+    int cc, n_count;          // channels of a chunk, counters
+    size_t xs, planes, vrange, slot, count, bytes;
+};
+
+static ClipLayout clip_layout(int C, int N, int d, int n_cand)
+{
+    ClipLayout l;
+    l.cc = clip_chunk_channels(C, d, n_cand);
+    const int chunks = (C + l.cc - 1) / l.cc;
+    const int last = (C - (chunks - 1) * l.cc) * n_cand, m_max = l.cc * n_cand;
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    l.xs = 256;
+    l.planes = l.xs + (size_t)N * d * 4;
+    l.vrange = l.planes + (size_t)m_max * d * 4;
+    l.slot = up(l.vrange + (size_t)m_max * 4);
+    l.count = l.slot + std::max(chunks > 1 ? clip_slot_bytes(clip_tiles(m_max), N) : 0,
+                                clip_slot_bytes(clip_tiles(last), N));
+    l.n_count = 2 * ((chunks - 1) * clip_tiles(m_max) + clip_tiles(last));
+    l.bytes = up(l.count + (size_t)l.n_count * 4);
+    return l;
+}
+
 size_t clip_f16_scratch_bytes(int C, int N, int d, int n_cand)
 {
-    const long long m_max = (long long)clip_chunk_channels(C, d, n_cand) * n_cand;
-    return 256 /* X range */ + (size_t)N * d * 4 /* X planes */ + (size_t)m_max * d * 4 /* planes */ +
-           ((size_t)m_max * 4 + 255) / 256 * 256 /* bounds */;
+    return clip_layout(C, N, d, n_cand).bytes;
 }
 
 mpq_status launch_clip_f16(const float *X, int N, const float *W, const float *clip,
                            const float *chmax, int C, int d, int qmax, int n_cand, float *err,
                            void *scratch, cudaStream_t stream)
 {
-    // scratch: the X range word, X's planes, the residual planes of one chunk, their bounds
-    const int cc = clip_chunk_channels(C, d, n_cand);
+    const ClipLayout l = clip_layout(C, N, d, n_cand);
+    const int cc = l.cc;
     char *p = static_cast<char *>(scratch);
     unsigned *xrange = reinterpret_cast<unsigned *>(p);
-    uint16_t *xs = reinterpret_cast<uint16_t *>(p + 256);
-    uint16_t *planes = reinterpret_cast<uint16_t *>(p + 256 + (size_t)N * d * 4);
-    unsigned *vrange = reinterpret_cast<unsigned *>(p + 256 + (size_t)N * d * 4 +
-                                                    (size_t)cc * n_cand * d * 4);
-    mpq_status st = launch_x_range(X, N, d, xrange, stream);
+    uint16_t *xs = reinterpret_cast<uint16_t *>(p + l.xs);
+    uint16_t *planes = reinterpret_cast<uint16_t *>(p + l.planes);
+    unsigned *vrange = reinterpret_cast<unsigned *>(p + l.vrange);
+    double *slot = reinterpret_cast<double *>(p + l.slot);
+    unsigned *count = reinterpret_cast<unsigned *>(p + l.count);
+    mpq_status st = launch_x_range(X, N, d, xrange, count, l.n_count, stream);
     if (st != MPQ_OK) return st;
     cudaError_t e = launch_x_split(X, N, d, xrange, xs, stream);
     if (e != cudaSuccess) return cuda_status(e, "X split kernel launch");
@@ -618,7 +654,8 @@ mpq_status launch_clip_f16(const float *X, int N, const float *W, const float *c
         st = cuda_status(e, "clip residual planes kernel launch");
         if (st == MPQ_OK)
             st = launch_clip_error(planes, N, M, d, err + (size_t)c0 * n_cand, xrange, vrange, xs,
-                                   stream);
+                                   count, slot, stream);
+        count += 2 * clip_tiles(M);
     }
     return st;
 }

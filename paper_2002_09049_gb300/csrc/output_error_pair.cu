@@ -333,10 +333,11 @@ mpq_status launch_output_error_pair(const float *X, int N, const float *W, const
     return MPQ_ERR_UNSUPPORTED;
 }
 
-mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, cudaStream_t stream)
+mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, unsigned *count,
+                          int n_count, cudaStream_t stream)
 {
     return cuda_status(launch_ranges<2>(X, N, nullptr, nullptr, nullptr, 0, d, false, range,
-                                        nullptr, 0, PadRows{nullptr, nullptr, 0}, stream),
+                                        count, n_count, PadRows{nullptr, nullptr, 0}, stream),
                        "X range pass");
 }
 

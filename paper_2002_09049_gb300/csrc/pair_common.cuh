@@ -63,8 +63,9 @@ __host__ __device__ inline bool tile_rows_ok(const float *X, const float *W, con
     return (d & 15) == 0 && (((uintptr_t)X | (uintptr_t)W | (uintptr_t)codes) & 15) == 0;
 }
 
-// Host: max|X| (float bits) into range[0], zeroed first.
-mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, cudaStream_t stream);
+// Host: max|X| (float bits) into range[0], zeroed first, and n_count zeros into count.
+mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, unsigned *count,
+                          int n_count, cudaStream_t stream);
 
 // Host: X * 2^e (e from xrange[0]) split into the fp16 hi and lo planes xs ([2][N][dp], dp = d
 // rounded up to 16, the rest of a row zero).
