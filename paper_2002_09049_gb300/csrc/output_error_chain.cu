@@ -529,7 +529,6 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
         mbar_init(&ctl.shared, E_VEC);
         ctl.abort = 0;
         ctl.any_slow = 0;
-        ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
         fence_barrier_init();
     }
     if (threadIdx.x < E_VEC) ctl.slow[threadIdx.x] = 0;
@@ -537,6 +536,8 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
         tmem_alloc_pair(&ctl.tmem_base, E_TMEM_COLS);
         tc_fence_before();
     }
+    griddep_wait();                     // nothing above reads global memory
+    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
     cluster_sync();                     // barriers of both CTAs initialised, TMEM allocated
     tc_fence_after();
     const uint32_t tmem = ctl.tmem_base;
@@ -1060,13 +1061,16 @@ mpq_status launch_chain(const float *X, const void *A, int N, const float *W, co
     cfg.blockDim = dim3(E_THREADS, 1, 1);
     cfg.dynamicSmemBytes = (size_t)G::SMEM;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    // (with fixed scratch the launches stay ordinary ones: a graph captured from them has no
+    // programmatic edges)
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1] = after_previous_kernel();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = RAWX ? 1 : 2;
     // one resident pair per two SMs (queried once per process), no more than units
     static std::atomic<int> resident{0};
     int pairs = resident.load(std::memory_order_relaxed);

@@ -144,13 +144,14 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
         }
         mbar_init(&ctl.done, 1);
         ctl.abort = 0;
-        ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
         fence_barrier_init();
     }
     if (warp == F_MMA_WARP) {
         tmem_alloc_pair(&ctl.tmem_base, F_TMEM_COLS);
         tc_fence_before();
     }
+    griddep_wait();                     // nothing above reads global memory
+    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
     cluster_sync();                     // barriers of both CTAs initialised, TMEM allocated
     tc_fence_after();
     const uint32_t tmem = ctl.tmem_base;
@@ -389,6 +390,8 @@ __global__ void __launch_bounds__(256)
 f16_split_kernel(const float4 *__restrict__ X, long long n8, const unsigned *__restrict__ xrange,
                  uint4 *__restrict__ hi, uint4 *__restrict__ lo)
 {
+    griddep_launch();
+    griddep_wait();
     const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += stride) {
@@ -409,6 +412,8 @@ f16_split_rows_kernel(const float *__restrict__ X, int N, int d, int dp,
                       const unsigned *__restrict__ xrange, uint4 *__restrict__ hi,
                       uint4 *__restrict__ lo)
 {
+    griddep_launch();
+    griddep_wait();
     const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
     const int d8 = dp / 8;
     const long long n8 = (long long)N * d8, stride = (long long)gridDim.x * blockDim.x;
@@ -453,6 +458,8 @@ clip_planes_kernel(const float *__restrict__ W, int d, const float *__restrict__
                    const float *__restrict__ chmax, int c0, int n_cand, int qmax, int M,
                    uint4 *__restrict__ hi, uint4 *__restrict__ lo, unsigned *__restrict__ vrange)
 {
+    griddep_launch();
+    griddep_wait();
     const int v = blockIdx.x, d8 = d / 8;
     if (v >= M) return;
     const long long k = c0 + v / n_cand;
@@ -541,13 +548,14 @@ mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
     cfg.blockDim = dim3(F_THREADS, 1, 1);
     cfg.dynamicSmemBytes = (size_t)F_SMEM;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1] = after_previous_kernel();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     // one resident pair per two SMs (queried once per process), no more than units
     static std::atomic<int> resident{0};
     int pairs = resident.load(std::memory_order_relaxed);
@@ -578,16 +586,18 @@ cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange,
     const int dp = (d + 15) / 16 * 16;
     const long long n8 = (long long)N * dp / 8;
     const int sb = (int)std::min<long long>((n8 + 255) / 256, 4LL * sm_count());
-    if (d != dp || ((uintptr_t)X & 15) != 0) {
-        f16_split_rows_kernel<<<(unsigned)std::max(sb, 1), 256, 0, stream>>>(
-            X, N, d, dp, xrange, reinterpret_cast<uint4 *>(xs),
-            reinterpret_cast<uint4 *>(xs + (size_t)N * dp));
-        return cudaGetLastError();
-    }
-    f16_split_kernel<<<(unsigned)std::max(sb, 1), 256, 0, stream>>>(
-        reinterpret_cast<const float4 *>(X), n8, xrange, reinterpret_cast<uint4 *>(xs),
-        reinterpret_cast<uint4 *>(xs + (size_t)N * d));
-    return cudaGetLastError();
+    cudaLaunchAttribute attr[1] = {after_previous_kernel()};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::max(sb, 1), 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    uint4 *hi = reinterpret_cast<uint4 *>(xs), *lo = reinterpret_cast<uint4 *>(xs + (size_t)N * dp);
+    if (d != dp || ((uintptr_t)X & 15) != 0)
+        return cudaLaunchKernelEx(&cfg, f16_split_rows_kernel, X, N, d, dp, xrange, hi, lo);
+    return cudaLaunchKernelEx(&cfg, f16_split_kernel, reinterpret_cast<const float4 *>(X), n8, xrange,
+                              hi, lo);
 }
 
 // Channels per chunk of residual planes: whole channels, at most 4 GiB of planes at a time.
@@ -648,9 +658,15 @@ mpq_status launch_clip_f16(const float *X, int N, const float *W, const float *c
         const int M = cn * n_cand;
         const int threads = std::min(128, (d / 8 + 31) / 32 * 32);
         uint4 *hi = reinterpret_cast<uint4 *>(planes);
-        clip_planes_kernel<<<(unsigned)M, (unsigned)threads, 0, stream>>>(
-            W, d, clip, chmax, c0, n_cand, qmax, M, hi, hi + (size_t)M * (d / 8), vrange);
-        e = cudaGetLastError();
+        cudaLaunchAttribute attr[1] = {after_previous_kernel()};
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)M, 1, 1);
+        cfg.blockDim = dim3((unsigned)threads, 1, 1);
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, clip_planes_kernel, W, d, clip, chmax, c0, n_cand, qmax, M, hi,
+                               hi + (size_t)M * (d / 8), vrange);
         st = cuda_status(e, "clip residual planes kernel launch");
         if (st == MPQ_OK)
             st = launch_clip_error(planes, N, M, d, err + (size_t)c0 * n_cand, xrange, vrange, xs,

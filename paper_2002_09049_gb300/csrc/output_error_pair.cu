@@ -20,6 +20,7 @@
 
 #include "mpq_internal.cuh"
 #include "pair_common.cuh"
+#include "sm100.cuh"
 
 MPQ_CHECKED_UNIT("output_error_pair.cu");
 
@@ -64,6 +65,7 @@ pair_range_kernel(const float *__restrict__ X, long long nx, int xb, int cb,
                   const PadRows pad)
 {
     constexpr int K = KP1 - 1;
+    sm100::griddep_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n_count; i += gridDim.x * 256) count[i] = 0u;
     if ((int)blockIdx.x < xb) {

@@ -42,6 +42,16 @@ __device__ __forceinline__ void split_f16x2(float a, float b, uint32_t &hi, uint
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
+// Host: launch attribute of a kernel that starts with griddep_wait and directly follows, on its stream,
+// a kernel of the same call.
+inline cudaLaunchAttribute after_previous_kernel()
+{
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+
 // Host: tile map over a row-major tensor (dims[0] contiguous, byte strides for dims 1..), zero
 // fill out of range, the given shared-memory swizzle.  False if the driver entry point is missing
 // or rejects the arguments.

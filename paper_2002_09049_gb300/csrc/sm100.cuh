@@ -347,6 +347,19 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
 
 // ---- TMA (bulk tensor copies global -> shared, completion counted on an mbarrier) ------------
 // Arms `bar` for `bytes` of incoming transactions and arrives once.
+// Programmatic dependent launch: griddep_launch lets the next kernel of the stream, if it was launched
+// for it, take SMs as they fall free; its griddep_wait returns once the kernels before it have
+// completed and what they wrote is visible (at once in a kernel launched the ordinary way).
+__device__ __forceinline__ void griddep_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void griddep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // 4 or 16 bytes from global to shared memory, asynchronously; only the first `bytes` are read, the
 // rest is zero.  cp_async_arrive: this thread's arrival on `bar` (in its count) once its copies so
 // far have landed.
