@@ -100,6 +100,17 @@ def test_bit_widths(gpu, oracle, bits):
     check(oracle, W, bits, 32, 3)
 
 
+# 8-bit codes on the lattice (up to 40,000 buckets where G <= 2 d) and just beyond either limit;
+# channel counts on both sides of the choice of warps per channel
+@pytest.mark.parametrize("C,d,G,k_max", [(9, 300, 128, 3), (40, 1456, 128, 1), (3, 64, 128, 2),
+                                         (3, 63, 128, 2), (4, 576, 157, 2), (4, 576, 158, 2),
+                                         (151, 96, 32, 2), (700, 200, 100, 2)])
+def test_long_lattices(gpu, oracle, C, d, G, k_max):
+    W = wlm.random_weights(C, d, C + d + G, "t")
+    rep = check(oracle, W, 8, G, k_max)
+    assert rep["near_ties"] <= max(1, C * k_max // 20)
+
+
 @pytest.mark.parametrize("G", [1, 2, 7, 31, 64, 128, 255, 256, 1024])
 def test_grid_sizes(gpu, oracle, G):
     W = wlm.random_weights(8, 130, 70 + G, "t")
