@@ -191,9 +191,29 @@ struct RingAt {
     }
 };
 
-// units: pairs of row tiles x input tiles; n_in: input tiles.
+// Work: (pair of row tiles, input tile) units, and after the first `full` of them parts of L_N / cut
+// inputs of the rest (lin_schedule).
+struct LinWork {
+    long long full, units;   // whole units, and units in all
+    int cut, n_in;           // parts of each of the rest; input tiles
+    struct Unit {
+        int tile, n0, width; // pair of row tiles, first input, inputs
+    };
+    __device__ __forceinline__ Unit at(long long u) const
+    {
+        long long v = u;
+        int part = 0, width = L_N;
+        if (u >= full) {
+            v = full + (u - full) / cut;
+            part = (int)((u - full) % cut);
+            width = L_N / cut;
+        }
+        return {(int)(v / n_in), (int)(v % n_in) * L_N + part * width, width};
+    }
+};
+
 __global__ void __launch_bounds__(L_THREADS, 1)
-multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int n_kc, int p,
+multipoint_linear_kernel(int T, int C, int tiles, const LinWork work, int n_kc, int p,
                          const int *__restrict__ coef, const int *__restrict__ chan,
                          const int *__restrict__ tile_R, const int *__restrict__ center_coef,
                          int32_t *__restrict__ Y, const WaitCtl wc,
@@ -210,9 +230,12 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int half = (int)cluster_ctarank();   // 0: even CTA (issues the MMAs), 1: its peer
-    // this pair's units pair0 + i n_pairs; unit u: row tiles 2 (u / n_in) + half, input tile u % n_in
+    // this pair's units pair0 + i n_pairs; this CTA has row tile 2 tile + half of each
     const int pair0 = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
-    const long long mine = (units - pair0 + n_pairs - 1) / n_pairs;
+    const long long mine = (work.units - pair0 + n_pairs - 1) / n_pairs;
+    auto width_of = [&](long long i) {   // inputs of this pair's unit i
+        return pair0 + i * n_pairs >= work.full ? L_N / work.cut : L_N;
+    };
     const long long chunks = mine * n_kc;
     if (!MPQ_CHECK_SMEM_END((size_t)pad + L_CTRL_BYTES + (size_t)L_BYTES)) return;
 
@@ -259,6 +282,7 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
         RingAt<L_SLOTS> at(grp);
         int kc = grp;   // chunk of the unit
         for (long long u = 0; u < mine && run; ++u, kc -= n_kc) {
+            const int rows = width_of(u) / 2;   // input rows of this CTA, 32 an item
             for (; kc < n_kc; kc += L_GROUPS) {
                 const int rs = ra.slot, sl = at.slot;
                 // (a fresh barrier's wait for the phase before its first returns at once)
@@ -277,13 +301,15 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
                 float4 raw[ITEMS];
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it)
-                    raw[it] = ld_shared_v4(x_u32 + rs * L_RAW_BYTES +
-                                           (uint32_t)(pt + it * L_GROUP_THREADS) * 16u);
+                    if (it * 32 < rows)
+                        raw[it] = ld_shared_v4(x_u32 + rs * L_RAW_BYTES +
+                                               (uint32_t)(pt + it * L_GROUP_THREADS) * 16u);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl.r_empty[rs]);
                 const uint32_t bb = b_u32 + sl * L_B_BYTES;
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it) {
+                    if (it * 32 >= rows) break;
                     const int q = pt + it * L_GROUP_THREADS;
                     const int row = q >> 2, c16 = q & 3;
                     const uint32_t w[4] = {__float_as_uint(raw[it].x), __float_as_uint(raw[it].y),
@@ -333,8 +359,9 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
                     int v = xs[it];
                     v += __shfl_xor_sync(0xffffffffu, v, 1);
                     v += __shfl_xor_sync(0xffffffffu, v, 2);
-                    int *at = &ctl.xsum[b][grp][half * L_IN + ((pt + it * L_GROUP_THREADS) >> 2)];
-                    if (run && (lane & 3) == 0) {
+                    const int row = (pt + it * L_GROUP_THREADS) >> 2;
+                    int *at = &ctl.xsum[b][grp][(half * rows + row) % L_N];
+                    if (run && (lane & 3) == 0 && row < rows) {
                         st_dsmem_u32(at, 0, (uint32_t)v);
                         st_dsmem_u32(at, 1, (uint32_t)v);
                     }
@@ -355,8 +382,9 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
             reinterpret_cast<int (*)[L_OUT_COLS + 1]>(ring + L_OFF_OUT) + ew * 32;
         const bool wide = (T & 3) == 0 && ((uintptr_t)Y & 15) == 0;   // 16-byte stores
         for (long long i = 0; i < mine; ++i) {
-            const long long u = pair0 + i * (long long)n_pairs;
-            const int tile = (int)(u / n_in) * 2 + half, n0 = (int)(u % n_in) * L_N + h * (L_N / 2);
+            const LinWork::Unit un = work.at(pair0 + i * (long long)n_pairs);
+            const int hw = un.width / 2;      // columns of a half
+            const int tile = un.tile * 2 + half, n0 = un.n0 + h * hw;
             const int b = (int)(i & 1);
             const bool real = tile < tiles;   // (an odd last tile's pair has no second one)
             const int R = real ? tile_R[tile] : 1;
@@ -375,13 +403,13 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
             if (__any_sync(0xffffffffu, !ok || *abort_flag)) break;   // warp-uniform
             tc_fence_after();
             const uint32_t lane_base =
-                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * L_N + h * (L_N / 2));
+                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * L_N + h * hw);
             // the rows this warp writes: one per channel (its first lane), -1 for none
             const int kw = (lane & (R - 1)) == 0 ? k : -1;
             ctl.kch[ew][lane] = kw;
             __syncwarp();
 #pragma unroll 1
-            for (int cb = 0; real && cb < L_N / 2 / 16 && n0 + cb * 16 < T; ++cb) {
+            for (int cb = 0; real && cb < hw / 16 && n0 + cb * 16 < T; ++cb) {
                 float v[16];
                 tmem_ld_32x32b_x16(lane_base + (uint32_t)(cb * 16), v);
                 long long sum[16];
@@ -392,8 +420,8 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
                     for (int j = 0; j < 16; ++j) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
                 }
                 if (centered) {   // the row sums first: no shared-memory store comes before them
-                    const int *xa = ctl.xsum[b][0] + h * (L_N / 2) + cb * 16;
-                    const int *xb = ctl.xsum[b][1] + h * (L_N / 2) + cb * 16;
+                    const int *xa = ctl.xsum[b][0] + h * hw + cb * 16;
+                    const int *xb = ctl.xsum[b][1] + h * hw + cb * 16;
 #pragma unroll
                     for (int j = 0; j < 16; ++j) sum[j] += ab * (long long)(xa[j] + xb[j]);
                 }
@@ -453,7 +481,8 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
     } else if (warp == L_MMA_WARP) {
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0 && half == 0) {
-            constexpr uint32_t idesc = idesc_bf16(2 * L_M, L_N);
+            uint32_t idesc = idesc_bf16(2 * L_M, width_of(0));
+            long long i = 0;
             int kc = 0;
             RingAt<2> acc;
             RingAt<L_SLOTS> at;
@@ -482,6 +511,7 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
                     mma_commit_pair(&ctl.acc_full[b], 3);
                     kc = 0;
                     acc.advance();
+                    idesc = idesc_bf16(2 * L_M, width_of(++i));
                 }
                 at.advance();
             }
@@ -496,7 +526,7 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
             prefetch_tensormap(&tmA);
             long long issued = 0;
             long long u = pair0;
-            int kc = 0, tile = (int)(u / n_in) * 2 + half;
+            int kc = 0, tile = work.at(u).tile * 2 + half;
             RingAt<L_SLOTS> aa;
             for (long long c = 0; c < chunks; ++c) {
                 const int as = aa.slot;
@@ -517,7 +547,7 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
                 if (++kc == n_kc) {
                     kc = 0;
                     u += n_pairs;
-                    tile = (int)(u / n_in) * 2 + half;
+                    tile = work.at(u).tile * 2 + half;
                 }
             }
             // no copy may land after the CTA is gone
@@ -531,7 +561,11 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
         if (lane == 0) {
             prefetch_tensormap(&tmX);
             long long issued = 0, u = pair0;
-            int kc = 0, n0 = (int)(u % n_in) * L_N + half * L_IN;
+            auto row0 = [&](long long v) {   // this CTA's first input row (a box holds a whole unit's)
+                const LinWork::Unit un = work.at(v);
+                return un.n0 + half * (un.width / 2);
+            };
+            int kc = 0, n0 = row0(u);
             RingAt<L_R_SLOTS> ra;
             for (long long c = 0; c < chunks; ++c) {
                 const int rs = ra.slot;
@@ -552,7 +586,7 @@ multipoint_linear_kernel(int T, int C, int tiles, long long units, int n_in, int
                 if (++kc == n_kc) {
                     kc = 0;
                     u += n_pairs;
-                    n0 = (int)(u % n_in) * L_N + half * L_IN;
+                    n0 = row0(u);
                 }
             }
             for (long long c = issued - L_R_SLOTS > 0 ? issued - L_R_SLOTS : 0; c < issued; ++c)
@@ -719,8 +753,33 @@ multipoint_mma_kernel(const int8_t *__restrict__ X, int T, int C, int d, int d_p
 // Which kernel takes a layer the tensor-memory kernel can take: the one whose modelled time is less,
 // in microseconds, fitted to both on layers of 64 x 576 to 11008 x 4096 with 1 to 2,048 inputs
 // (within some 15 %).  Here: waves of resident blocks, each a fixed cost and one per K chunk; there:
-// a fixed cost and 0.45 us per chunk of every round of units.  4096 x 4096 at 8 / 64 / 128 / 256 /
-// 2,048 inputs: 7.4 / 25.6 / 38.7 / 66.5 / 485 us here, 32.9 / 34.7 / 37.0 / 39.6 / 104 there.
+// a fixed cost and lin_schedule's time of a chunk over the rounds.  4096 x 4096 at 8 / 64 / 128 / 256 /
+// 2,048 inputs: 7.4 / 25.6 / 38.7 / 66.5 / 485 us here, 32.9 / 34.7 / 37.0 / 34.5 / 98 there.
+struct LinSchedule {
+    long long full, units;
+    int cut;
+    double chunk_us;   // modelled time of a K chunk, over the rounds
+};
+
+// The last round of units leaves pairs idle: what is beyond whole rounds is cut into 1, 2 or 4 parts
+// by its inputs, whichever takes the least.  A chunk of a half or quarter takes 0.36 and 0.35 us: its
+// codes tile and hand-overs stay (a smaller box for its inputs changes nothing).  4096 x 4096 at 256 /
+// 1,024 / 2,048 inputs (21, 84, 168 units on 76 pairs) 39.4 / 72.6 / 105 -> 34.5 / 65 / 98 us, 11008 x
+// 4096 at 512 73.5 -> 67.8.
+LinSchedule lin_schedule(long long units, long long pairs)
+{
+    const double part_us[3] = {0.45, 0.36, 0.35};
+    const long long rest = units % pairs;
+    LinSchedule s = {units, units, 1, part_us[0] * (double)((units + pairs - 1) / pairs)};
+    for (int i = 1; i < 3 && rest > 0; ++i) {
+        const int cut = 1 << i;
+        const double t = part_us[0] * (double)(units / pairs) +
+                         part_us[i] * (double)((rest * cut + pairs - 1) / pairs);
+        if (t < s.chunk_us) s = {units - rest, units - rest + rest * cut, cut, t};
+    }
+    return s;
+}
+
 bool few_inputs(const mpq_packed_layout *L, int T)
 {
     const double n_kc = L->d_pad / L_KC, sms = sm_count();
@@ -734,9 +793,9 @@ bool few_inputs(const mpq_packed_layout *L, int T)
         per_sm = 2.0;
         wave = 4.5 + 0.15 * n_kc;
     }
-    const double units = (L->tiles + 1) / 2 * floor((T + (double)L_N - 1) / L_N);
+    const long long units = (L->tiles + 1LL) / 2 * (((long long)T + L_N - 1) / L_N);
     const double here = ceil(blocks / (per_sm * sms)) * wave;
-    const double there = 10.0 + 0.45 * n_kc * ceil(units / (sms / 2));
+    const double there = 10.0 + n_kc * lin_schedule(units, std::max(1, sm_count() / 2)).chunk_us;
     return here <= there;
 }
 
@@ -945,10 +1004,13 @@ mpq_status launch_multipoint_linear(const int8_t *X, int T, const mpq_packed_lay
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         // one resident pair per two SMs, no more than units
-        const long long pairs = std::min<long long>(std::max(1, sm_count() / 2), units);
+        const long long resident = std::max(1, sm_count() / 2);
+        const LinSchedule sch = lin_schedule(units, resident);
+        const LinWork work = {sch.full, sch.units, sch.cut, (int)n_in};
+        const long long pairs = std::min<long long>(resident, sch.units);
         cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
         const cudaError_t el =
-            cudaLaunchKernelEx(&cfg, multipoint_linear_kernel, T, L->C, L->tiles, units, (int)n_in,
+            cudaLaunchKernelEx(&cfg, multipoint_linear_kernel, T, L->C, L->tiles, work,
                                L->d_pad / L_KC, L->p, (const int *)v.coef, (const int *)v.chan,
                                (const int *)v.tile_R, (const int *)v.center, Y, wc, tmA, tmX);
         if (el != cudaSuccess) return cuda_status(el, "multipoint linear kernel launch");

@@ -131,7 +131,9 @@ def test_few_inputs_and_odd_rows(gpu, oracle, d, bits, off, T):
 
 
 @pytest.mark.parametrize("C,d,T", [(3100, 64, 1024), (40, 1088, 3000), (2100, 320, 514),
-                                   (1500, 448, 777)])
+                                   (1500, 448, 777),
+                                   # the last round cut by its inputs into 2 and 4 parts
+                                   (200, 256, 520), (5200, 64, 1000), (700, 128, 513), (3000, 192, 600)])
 def test_pairs_and_rounds(gpu, oracle, C, d, T):
     """The tensor-memory kernel: an odd number of row tiles, a second round of units, inputs not a
     multiple of 4 (no 16-byte stores) or of 256, one chunk a unit, with centres."""
