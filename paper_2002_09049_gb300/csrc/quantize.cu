@@ -484,8 +484,10 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
             if (MPQ_IN((g + 1) * (2 * L - 1), nb)) lut[(g + 1) * (2 * L - 1)] = 1;
         }
         __syncthreads();
-        // inclusive count of positions, minus one: a contiguous block of buckets per thread
-        const int per = (nb + QTHREADS - 1) / QTHREADS;
+        // inclusive count of positions, minus one: a contiguous block of buckets per thread, an odd
+        // number of words (64 or 128 buckets would put every lane on one bank: 8-bit codes, G = 64,
+        // 35 us of set-up a CTA; 13 so)
+        const int per = 2 * ((nb + 2 * QTHREADS - 1) / (2 * QTHREADS) | 1);
         const int b0 = min(nb, (int)threadIdx.x * per), b1 = min(nb, b0 + per);
         int own = 0;
         for (int b = b0; b < b1; ++b) own += lut[b];
@@ -917,9 +919,39 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                     }
                     gsync<WPC>(grp);
                 }
-                // ---- the decision, every candidate in double (two bounded fp32 passes before it cost
-                // more: 64 channels x 576 lost 0.5 us a step to their barriers)
+                // ---- the decision in double.  Groups of 4 and 8 warps decide every candidate (bounded
+                // fp32 passes before it cost more: 64 channels x 576 lost 0.5 us a step to their
+                // barriers).  With fewer warps and 4 or more candidates a thread, an SM has more channels
+                // and the double rate bounds them (6168 x 219, 3 bits, G = 256: 124 us, screened
+                // 97): each warp keeps the candidates whose error interval can contain its own
+                // minimum, D / 2^2e = s'(s'N - 2P') in fp32 with s' = s / 2^e and P' = P 2^-S / 2^e
+                // (both O(1); at most ~8 roundings of 2^-24, the bound allows 2^-20).
+                float upper = FLT_MAX, pscale = 0.0f, smax_e = 0.0f;
+                auto screened = [&](int g, float &err) {
+                    const float sh = fg(g) * smax_e;
+                    const float Nf = (float)(int)(Nbase + mN[g + 1]);
+                    const float Pf = __ll2float_rn(Pbase + bin64(mLo, mHi, g + 1)) * pscale;
+                    err = sh * (sh * Nf + 2.0f * Pf) * MPQ_FAST_REL;
+                    return sh * (sh * Nf - 2.0f * Pf);
+                };
+                const bool screen = WPC <= 2 && G >= 4 * NT;
+                if (screen) {
+                    pscale = ldexpf(1.0f, -S - e);
+                    smax_e = ldexpf(smax, -e);
+                    for (int g = gt; g < G; g += NT) {
+                        float err;
+                        const float D32 = screened(g, err);
+                        upper = fminf(upper, D32 + err);
+                    }
+                    for (int o = 16; o > 0; o >>= 1)
+                        upper = fminf(upper, __shfl_xor_sync(0xffffffffu, upper, o));
+                }
                 for (int g = gt; g < G; g += NT) {
+                    if (screen) {
+                        float err;
+                        const float D32 = screened(g, err);
+                        if (!(D32 - err <= upper)) continue;
+                    }
                     const double D = decision(__fmul_rn(fg(g), smax), Pbase + bin64(mLo, mHi, g + 1),
                                               Nbase + mN[g + 1], down);
                     if (D < bestD) {
@@ -1247,14 +1279,21 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
     const long long smem_cap = max_smem_optin();
     // Lattice form on the linear grid when a bucket's fields fit one word, and the lattice is small
     // or (its per-step cost is O(G Qmax), the event form's O(d) times the levels crossed) the row is
-    // long for it and it still fits: 64 x 576 with 8-bit codes and G = 64, 333 -> 80 us.
+    // long for it and it still fits.  The event form has a long step (45 us with 8-bit codes) that
+    // many channels share, the lattice form a short one with few channels on an SM, so where there
+    // are many channels the row has to be longer.  8-bit codes, G = 64 (16,257 buckets), k_max = 6,
+    // event -> lattice form, us: 64 x 576 333 -> 80; 1500 x 100 466 -> 474, x 200 849 -> 485; 4000 x
+    // 130 1081 -> 1304, x 200 1543 -> 1322.  5 bits, G = 256 (7,681): 4000 x 130 285 -> 325, x 200 374 -> 328.
     LatBits lb;
     const long long nb_all = (long long)2 * G * qmax + 1;
     bool lat = !CUSTOM && nb_all <= 40000 && lattice_bits(d, qmax, G, &lb);
     if (lat) {
         lb.nc = lattice_positions(G, qmax);
+        const long long shortest = C > 16LL * sm_count()  ? nb_all / 50
+                                   : C > 4LL * sm_count() ? nb_all / 70
+                                                          : 0;
         if (nb_all > 4096)
-            lat = G <= 2 * d && (long long)(group_words(G, d, 1, lb.nc) * 4 + table_bytes(G) +
+            lat = G <= 2 * d && d >= shortest && (long long)(group_words(G, d, 1, lb.nc) * 4 + table_bytes(G) +
                                             lut_bytes((int)nb_all)) <= smem_cap;
     }
     if (!lat) lb = LatBits{0, 31, 0};
@@ -1262,13 +1301,13 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
     const int nc = lb.nc;
     const size_t per_group = group_words(G, d, 1, nc) * 4;
     // Warps per channel.  A step's fixed work (scans, fold, decision, barriers) grows with the warps
-    // of a channel, so no more of them than fill the GPU to about 27 warps an SM (1280 x 320: 2
-    // warps 58 us, 4 warps 96), at least ~16 elements per warp (candidates, on rows evaluated
+    // of a channel, so no more of them than leave every channel resident at once, 32 warps an SM
+    // (1280 x 320: 2 warps 58 us, 4 warps 96; 2281 x 128, G = 100: 1 warp 103, 2 warps 88), at least ~16 elements per warp (candidates, on rows evaluated
     // directly), at least 4 warps for rows of 1,024 and more (4096 x 1024, G = 256: 200 us against
     // 323 with 2), and enough warps per SM (24) for the shared memory the channels need -- on
     // layers with thousands of long channels, 4-warp groups (more channels per SM, barriers over
     // fewer warps) measured faster than 8-warp ones (11008 x 4096: 1.51 ms against 1.94).
-    const long long warps_gpu = (long long)sm_count() * 27;
+    const long long warps_gpu = (long long)sm_count() * 32;
     int wpc_c = 1;
     while (wpc_c < 8 && (long long)C * wpc_c * 2 <= warps_gpu) wpc_c *= 2;
     int wpc_e = 1;
