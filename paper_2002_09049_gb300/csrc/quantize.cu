@@ -234,7 +234,9 @@ __device__ __forceinline__ void group_suffix_scan(int t0, int t1, Load load, Sto
     constexpr int NT = WPC * 32;
     const int gt = gw * 32 + lane;
     const int n = t1 - t0;
-    const int per = (n + NT - 1) / NT;
+    // odd: the lanes' blocks start on different banks (4000 to 11008 channels, G = 256, even blocks of
+    // 8 to 40: 8000 x 64 448 -> 211 us, 6315 x 384 381 -> 191, 11008 x 4096 1406 -> 1298)
+    const int per = ((n + NT - 1) / NT) | 1;
     const int b0 = t0 + min(n, gt * per), b1 = t0 + min(n, gt * per + per);
     unsigned long long sp = 0;
     long long sn = 0;
@@ -290,7 +292,7 @@ __device__ __forceinline__ void warps_suffix_scan(int t0, int t1, Load load, Sto
 {
     const int nt = nw * 32, st = sw * 32 + lane;
     const int n = t1 - t0;
-    const int per = (n + nt - 1) / nt;
+    const int per = ((n + nt - 1) / nt) | 1;   // odd: the lanes' blocks start on different banks
     const int b0 = t0 + min(n, st * per), b1 = t0 + min(n, st * per + per);
     unsigned long long sp = 0;
     long long sn = 0;
@@ -923,7 +925,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                 // fp32 passes before it cost more: 64 channels x 576 lost 0.5 us a step to their
                 // barriers).  With fewer warps and 4 or more candidates a thread, an SM has more channels
                 // and the double rate bounds them (6168 x 219, 3 bits, G = 256: 124 us, screened
-                // 97): each warp keeps the candidates whose error interval can contain its own
+                // 97, and 78 with the scans as they are): each warp keeps the candidates whose error interval can contain its own
                 // minimum, D / 2^2e = s'(s'N - 2P') in fp32 with s' = s / 2^e and P' = P 2^-S / 2^e
                 // (both O(1); at most ~8 roundings of 2^-24, the bound allows 2^-20).
                 float upper = FLT_MAX, pscale = 0.0f, smax_e = 0.0f;
@@ -1302,7 +1304,7 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
     const size_t per_group = group_words(G, d, 1, nc) * 4;
     // Warps per channel.  A step's fixed work (scans, fold, decision, barriers) grows with the warps
     // of a channel, so no more of them than leave every channel resident at once, 32 warps an SM
-    // (1280 x 320: 2 warps 58 us, 4 warps 96; 2281 x 128, G = 100: 1 warp 103, 2 warps 88), at least ~16 elements per warp (candidates, on rows evaluated
+    // (1280 x 320: 2 warps 55 us, 4 warps 82; 1500 x 128, G = 100: 1 warp 47, 2 warps 38), at least ~16 elements per warp (candidates, on rows evaluated
     // directly), at least 4 warps for rows of 1,024 and more (4096 x 1024, G = 256: 200 us against
     // 323 with 2), and enough warps per SM (24) for the shared memory the channels need -- on
     // layers with thousands of long channels, 4-warp groups (more channels per SM, barriers over
