@@ -1377,8 +1377,8 @@ def run_adaptive(args, world, rank, local):
     alu_peak = sms * ALU_LANES_PER_SM * mhz * 1e6 / 1e12
     ach = sum(adaptive_ops(wl, l) for l in layers) / t1 / 1e12
     roofline = {"kernel": "adaptive_kernel (Algorithm 1 over the grid of Eq. 10: code-level "
-                          "thresholds sorted, piecewise quadratic screened in fp32, settled in "
-                          "double)", "bound": "alu", "achieved": ach, "peak": alu_peak,
+                          "thresholds screened by buckets, the rest sorted, piecewise quadratic "
+                          "settled in double)", "bound": "alu", "achieved": ach, "peak": alu_peak,
                 "unit": "Tlane-op/s", "frac": ach / alu_peak, "traffic": None,
                 "peak_source": f"{sms} SMs x {ALU_LANES_PER_SM} lanes x {mhz:.0f} MHz; "
                                f"{ADAPTIVE_OPS_PER_THRESHOLD} lane operations per code-level "

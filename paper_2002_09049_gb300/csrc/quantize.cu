@@ -1311,13 +1311,20 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
     // fewer warps) measured faster than 8-warp ones (11008 x 4096: 1.51 ms against 1.94).
     const long long warps_gpu = (long long)sm_count() * 32;
     int wpc_c = 1;
-    while (wpc_c < 8 && (long long)C * wpc_c * 2 <= warps_gpu) wpc_c *= 2;
+    // The event form's step is its elements', which more warps share: as many as fill the GPU, at
+    // least 2 elements per lane (1396 x 912, 8 bits, G = 128 on a caller's grid: 3.54 ms by the lines
+    // above, 3.34 so).
+    const bool event = !lat && d > QDIRECT_MAX_D;
+    while (wpc_c < 8 && (event ? (long long)C * wpc_c < warps_gpu : (long long)C * wpc_c * 2 <= warps_gpu))
+        wpc_c *= 2;
     int wpc_e = 1;
-    if (d <= QDIRECT_MAX_D) wpc_e = G >= 64 ? 2 : 1;
+    if (event)
+        while (wpc_e < 8 && wpc_e * 64 <= d) wpc_e *= 2;
+    else if (d <= QDIRECT_MAX_D) wpc_e = G >= 64 ? 2 : 1;
     else
         while (wpc_e < 8 && wpc_e * 16 <= d) wpc_e *= 2;
     const long long groups_per_sm = (long long)(227 * 1024) / (long long)(per_group + 256);
-    int wpc_s = d >= 1024 ? 4 : 1;
+    int wpc_s = d >= 1024 && !event ? 4 : 1;
     while (wpc_s < 8 && groups_per_sm * wpc_s < 24) wpc_s *= 2;
     int wpc = wpc_c < wpc_e ? wpc_c : wpc_e;
     if (wpc < wpc_s) wpc = wpc_s;
