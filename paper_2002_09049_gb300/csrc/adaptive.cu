@@ -383,7 +383,8 @@ struct AShared {
     unsigned skey;              // its scale's bits, among equal D
     double U;                   // best exact D of the first settled piece
     int state;                  // 0 search, 1 scale 0 (null point or no positive grid scale), 2 dead
-    int nev;
+    int nev;                    // candidate thresholds of the step
+    int nall;                   // adaptive_search_all's count: nev still decides the branch to it
     float spos, slast;
     float amax[AW];             // max |r| per warp
     float gsmall[AW];
@@ -703,14 +704,13 @@ __device__ __forceinline__ float ad_search_pieces(const AStep &q, AShared &sh, i
 }
 
 // Every threshold at or above the grid's first positive scale, sorted in global scratch (bufA,
-// bufB: cap entries each): for rows whose candidate thresholds do not fit the sort list.
+// bufB: cap entries each): for rows whose candidate thresholds do not fit the sort list.  Workers
+// enter one by one: a word that the branch to it reads (sh.nev) must not change here.
 __device__ __noinline__ float adaptive_search_all(const AStep &q, AShared &sh, uint2 *bufA,
                                                   uint2 *bufB, int cap)
 {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const float *r = q.r;
-    if (t == 0) sh.nev = 0;
-    ad_sync();
     long long P0 = 0, N0 = 0;   // totals: P and N at spos (every kept threshold is held there)
     for (int j = t; j < q.d; j += AT) {
         const float a = fabsf(r[j]);
@@ -719,7 +719,7 @@ __device__ __noinline__ float adaptive_search_all(const AStep &q, AShared &sh, u
         for (int L = 1; L <= q.qmax; ++L) {
             const float tau = ad_threshold(a, L);
             if (!(tau >= q.spos)) break;   // tau is non-increasing in L
-            const int pos = atomicAdd(&sh.nev, 1);
+            const int pos = atomicAdd(&sh.nall, 1);
             if (MPQ_IN(pos, cap))
                 bufA[pos] = make_uint2(__float_as_uint(tau), ((unsigned)j << 8) | (unsigned)L);
             P0 += R;
@@ -743,7 +743,7 @@ __device__ __noinline__ float adaptive_search_all(const AStep &q, AShared &sh, u
         N0 += sh.part[x][1];
     }
     ad_sync();
-    int n = sh.nev;
+    int n = sh.nall;
     if (!MPQ_CHECK(n <= cap)) n = cap;
     const uint2 *ev = ad_sort(bufA, bufB, n, sh.sort);
     // pieces e = 0..n: scales (lo, hi] with the first e thresholds passed
@@ -897,6 +897,7 @@ adaptive_kernel(const float *__restrict__ W, int C, int d, int qmax, int k_max, 
                     sh.skey = ~0u;
                     sh.nlist = 0;
                     sh.nev = 0;
+                    sh.nall = 0;
                 }
                 float amax = 0.0f;
                 for (int x = 0; x < AW; ++x) amax = fmaxf(amax, sh.amax[x]);

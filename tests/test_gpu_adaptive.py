@@ -128,13 +128,12 @@ def test_adaptive_tiny_gap_zero_scales(gpu, oracle):
 @pytest.mark.parametrize("C,d,bits,k_max,kind", [
     (4, 73, 4, 2, "normal"),      # 511 thresholds: all of them listed
     (4, 74, 4, 2, "normal"),      # 518: counted in buckets first
-    (3, 640, 4, 2, "lattice"),    # equal magnitudes by the hundred: the sort list overflows
+    (3, 640, 4, 2, "lattice"),    # equal magnitudes by the hundred, many in one bucket
     (3, 700, 3, 2, "binades"),    # magnitudes over 24 binades, ties in the norm's additions
     (2, 130, 7, 2, "tails"),      # Qmax = 63 and outliers: scales far below the largest weight
 ])
 def test_adaptive_bucket_screen(gpu, oracle, C, d, bits, k_max, kind):
-    """The bucket screen's edges: row lengths on both sides of its rule, rows whose candidate
-    thresholds do not fit the sort list, wide ranges of magnitudes."""
+    """The bucket screen's edges: row lengths on both sides of its rule, wide ranges of magnitudes."""
     rng = np.random.default_rng(d)
     W = rng.standard_normal((C, d)).astype(np.float32)
     if kind == "lattice":
@@ -144,3 +143,15 @@ def test_adaptive_bucket_screen(gpu, oracle, C, d, bits, k_max, kind):
     elif kind == "tails":
         W = np.where(rng.random((C, d)) < 0.02, W * 300, W).astype(np.float32)
     check(oracle, W, bits, k_max, cap=BIG, piecewise=True)
+
+
+def test_adaptive_overflowing_lists(gpu, oracle):
+    """More candidate thresholds than the sort list holds (2,048), several channels a CTA: the
+    workers all take the branch to the full sort, whichever comes first.  2,200 elements of
+    magnitude a end their code 1 at s = 2 a, just above the best scale that 5,600 elements of
+    14 a = 7 * 2 a ask for: one bucket with 2,200 thresholds that no bound can leave out."""
+    rng = np.random.default_rng(7800)
+    a = np.exp2(rng.integers(-6, -3, (350, 1))) * rng.uniform(1.0, 1.9, (350, 1))
+    W = np.concatenate([np.ones((350, 2200)), np.full((350, 5600), 14.0)], axis=1) * a
+    W = rng.permuted(W * rng.choice([-1.0, 1.0], W.shape), axis=1).astype(np.float32)
+    check(oracle, W, 4, 2, cap=BIG, piecewise=True, sample=np.arange(0, 350, 25))
