@@ -299,7 +299,8 @@ mpq_status mpq_center_weights(const float *W, int C, int d, int mode, float *cen
  * NaN, and NaN never wins; best is -1 where no candidate is finite.
  *
  *   X, N, groups  calibration inputs as for mpq_output_error.
- *   W, C, d       [C][d] fp32 weights; 1 <= d <= MPQ_MAX_DIM.
+ *   W, C, d       [C][d] fp32 weights; 1 <= d <= MPQ_MAX_DIM (with groups == C: MPQ_ERR_UNSUPPORTED
+ *                 beyond the 8 rows of d floats that shared memory holds, d <= 7256 on GB300).
  *   bits          b in [MPQ_MIN_BITS, MPQ_MAX_BITS].
  *   n_cand        1..MPQ_MAX_CLIP_CANDIDATES.
  *   mode          MPQ_CLIP_PER_CHANNEL or MPQ_CLIP_PER_LAYER.

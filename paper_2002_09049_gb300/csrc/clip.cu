@@ -435,11 +435,6 @@ mpq_status launch_clip(const float *X, int N, int groups, const float *W, int C,
         if (st != MPQ_OK) return st;
     } else {
         if (e != cudaSuccess) return cuda_status(e, "clip candidate kernel launch");
-        const size_t smem = (size_t)CL_CHUNK * d * sizeof(float);
-        if ((long long)smem > max_smem_optin()) {
-            set_error("clip search with d = %d needs %zu bytes of shared memory", d, smem);
-            return MPQ_ERR_UNSUPPORTED;
-        }
         if (groups == 1) {
             // the rows a thread and the split of the row tiles over a cluster's CTAs with the least
             // work on one SM, a chunk costing R products and about 4 more's time for its residuals
@@ -478,6 +473,11 @@ mpq_status launch_clip(const float *X, int N, int groups, const float *W, int C,
                                                      : clip_rows_kernel<2>, X, N, W, C, d, qmax, n_cand,
                                    (const float *)clip, err);
         } else {
+            const size_t smem = (size_t)CL_CHUNK * d * sizeof(float);
+            if ((long long)smem > max_smem_optin()) {
+                set_error("clip search with d = %d needs %zu bytes of shared memory", d, smem);
+                return MPQ_ERR_UNSUPPORTED;
+            }
             e = cudaFuncSetAttribute(clip_errors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem);
             if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");

@@ -46,7 +46,9 @@ def test_shared_input(gpu, oracle, mode, C, d, N, n_cand):
                                               (13, 31, 128, 5, 0), (1, 1, 1, 1, 0),
                                               (7, 147, 1025, 32, 0), (2, 33, 5000, 20, 0),
                                               (300, 75, 260, 20, 0), (5, 64, 300, 20, 1),
-                                              (5, 50, 300, 3, 3)])
+                                              (5, 50, 300, 3, 3),
+                                              # rows longer than per-channel inputs can have
+                                              (2, 8191, 40, 3, 0), (2, 7280, 40, 3, 1)])
 def test_rows_of_any_length(gpu, oracle, C, d, N, n_cand, off):
     W = wlm.random_weights(C, d, C + d + N, "laplace")
     X = wlm.random_calibration(N, d, 7 + N)
