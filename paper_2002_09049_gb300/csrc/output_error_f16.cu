@@ -446,8 +446,11 @@ f16_split_rows_kernel(const float *__restrict__ X, int N, int d, int dp,
 
 // Clipping search (Eq. 12): the residual r = w - s q of channel c0 + v / n_cand under candidate
 // v mod n_cand (s = K / Qmax, the codes q of Eq. 8 with the sign of w, q = 0 where s is 0 or NaN),
-// scaled by 2^e and split into fp16 hi/lo planes ([2][M][d] as hi and lo).  One CTA per vector v,
-// 8 elements a thread per step.  e comes from a bound on the vector's elements,
+// scaled by 2^e and split into fp16 hi/lo planes ([2][M][d] as hi and lo).  A CTA takes vectors a
+// grid apart, 8 elements a thread per step: one vector each would make CTAs that live for a few loads,
+// and each of them pays for the dependent launch's instructions (65,536 vectors of 64 elements, 32
+// candidates, N = 128, the whole call: 104 us, 73 without those instructions, 58 so; 20,000 of 2,048
+// the same either way).  e comes from a bound on the vector's elements,
 // max(min(max|w|, s/2), max|w| - Qmax s): an element with code 0 keeps r = w, one with a nearest
 // nonzero code |r| <= s/2, a clamped one |r| = |w| - Qmax s (a residual a rounding above the bound
 // still fits fp16, whose range reaches 2^16); kept in vrange[v] (float bits) for the contraction.
@@ -460,38 +463,39 @@ clip_planes_kernel(const float *__restrict__ W, int d, const float *__restrict__
 {
     griddep_launch();
     griddep_wait();
-    const int v = blockIdx.x, d8 = d / 8;
-    if (v >= M) return;
-    const long long k = c0 + v / n_cand;
+    const int d8 = d / 8;
     const float qmaxf = (float)qmax, qlim = qmaxf + 1.0f;
     const float tband = 0.5f - MPQ_FAST_REL * (qlim + 1.0f);
-    // clip row of channel k, candidate v mod n_cand: index c0 n_cand + v
-    const float sv = __fdiv_rn(__ldg(clip + (long long)c0 * n_cand + v), qmaxf);
-    const float inv = sv > 0.0f ? __frcp_rn(sv) : 0.0f;
-    const float m = __ldg(chmax + k);
-    const float bound = fmaxf(fminf(m, __fmul_rn(0.5f, sv)), __fmaf_rn(-qmaxf, sv, m));
-    const float vf = pow2f(f16_scale_exp(bound));
-    if (threadIdx.x == 0) vrange[v] = __float_as_uint(bound);
-    const float4 *w4 = reinterpret_cast<const float4 *>(W + k * d);
-    const long long row = (long long)v * d8;
-    for (int j = threadIdx.x; j < d8; j += blockDim.x) {
-        const float4 a = __ldg(w4 + 2 * j), b = __ldg(w4 + 2 * j + 1);
-        const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        float q[8];
-        bool unsure = false;
+    for (int v = blockIdx.x; v < M; v += gridDim.x) {
+        const long long k = c0 + v / n_cand;
+        // clip row of channel k, candidate v mod n_cand: index c0 n_cand + v
+        const float sv = __fdiv_rn(__ldg(clip + (long long)c0 * n_cand + v), qmaxf);
+        const float inv = sv > 0.0f ? __frcp_rn(sv) : 0.0f;
+        const float m = __ldg(chmax + k);
+        const float bound = fmaxf(fminf(m, __fmul_rn(0.5f, sv)), __fmaf_rn(-qmaxf, sv, m));
+        const float vf = pow2f(f16_scale_exp(bound));
+        if (threadIdx.x == 0) vrange[v] = __float_as_uint(bound);
+        const float4 *w4 = reinterpret_cast<const float4 *>(W + k * d);
+        const long long row = (long long)v * d8;
+        for (int j = threadIdx.x; j < d8; j += blockDim.x) {
+            const float4 a = __ldg(w4 + 2 * j), b = __ldg(w4 + 2 * j + 1);
+            const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            float q[8];
+            bool unsure = false;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) q[e] = code_signed_fast(w[e], inv, qmaxf, qlim, tband, unsure);
-        if (unsure) {
+            for (int e = 0; e < 8; ++e) q[e] = code_signed_fast(w[e], inv, qmaxf, qlim, tband, unsure);
+            if (unsure) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) q[e] = code_signed_exact(w[e], sv, qmaxf);
+                for (int e = 0; e < 8; ++e) q[e] = code_signed_exact(w[e], sv, qmaxf);
+            }
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                split_f16x2(__fmul_rn(__fmaf_rn(-sv, q[2 * e], w[2 * e]), vf),
+                            __fmul_rn(__fmaf_rn(-sv, q[2 * e + 1], w[2 * e + 1]), vf), h[e], l[e]);
+            hi[row + j] = make_uint4(h[0], h[1], h[2], h[3]);
+            lo[row + j] = make_uint4(l[0], l[1], l[2], l[3]);
         }
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            split_f16x2(__fmul_rn(__fmaf_rn(-sv, q[2 * e], w[2 * e]), vf),
-                        __fmul_rn(__fmaf_rn(-sv, q[2 * e + 1], w[2 * e + 1]), vf), h[e], l[e]);
-        hi[row + j] = make_uint4(h[0], h[1], h[2], h[3]);
-        lo[row + j] = make_uint4(l[0], l[1], l[2], l[3]);
     }
 }
 
@@ -660,7 +664,7 @@ mpq_status launch_clip_f16(const float *X, int N, const float *W, const float *c
         uint4 *hi = reinterpret_cast<uint4 *>(planes);
         cudaLaunchAttribute attr[1] = {after_previous_kernel()};
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)M, 1, 1);
+        cfg.gridDim = dim3((unsigned)std::min(M, 32 * sm_count()), 1, 1);
         cfg.blockDim = dim3((unsigned)threads, 1, 1);
         cfg.stream = stream;
         cfg.attrs = attr;

@@ -31,6 +31,8 @@ def run_both(oracle, X, W, bits, n_cand, mode, groups=1):
     # d % 16 == 0: CTA-pair tensor-core path -- several pair tiles, a part-filled odd CTA, ragged
     # row tiles split over clusters, 1 to 32 candidates
     (50, 256, 600, 20), (13, 64, 100, 32), (130, 128, 300, 7), (3, 48, 20, 1), (64, 576, 512, 20),
+    # more residual vectors than CTAs that write their planes
+    (700, 16, 33, 20),
     # other rows: fp32 register tiles
     (11, 147, 129, 20), (4, 33, 70, 5), (2, 17, 300, 32),
 ])
