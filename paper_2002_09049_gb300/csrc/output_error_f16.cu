@@ -501,18 +501,39 @@ clip_planes_kernel(const float *__restrict__ W, int d, const float *__restrict__
 
 int clip_tiles(int vectors) { return (vectors + 2 * F_VEC - 1) / (2 * F_VEC); }
 
-// Parts of a vector tile's row tiles: single row tiles up to about 16 units a pair, larger parts
-// beyond (the scratch of their sums stays below about 5 MB), never more than row tiles.
-int clip_parts(int tiles, int N)
+// Parts of a vector tile's row tiles, each one unit: those with the least modelled time on the busiest
+// pair, in twentieths of a step of 64 elements -- a row tile costs its steps (a twentieth more where
+// the planes of the vector tiles at work do not stay in L2 from one row tile to the next: 1746 x 1920,
+// N = 2020, 32 candidates 820 us whole, 790 in 3 parts, as many row tiles a pair), the end of a unit
+// two (its sums, which nothing of the pair overlaps), leaving them to another pair half a step more.
+// Fewer parts on ties; at most about 16 units a pair (the scratch of their sums stays below about 5 MB),
+// never more than row tiles.  Single row tiles throughout cost short rows dearly: 2048 x 64, N = 2048,
+// 20 candidates 139 us in 8 parts, 89 whole; 1000 x 2048 338 us in 8 parts, 540 whole.  Fitted to 126
+// layers of 64 to 2,048 channels, 64 to 2,048 elements and 500 to 2,048 rows (within 2 % on average).
+int clip_parts(int tiles, int N, int d)
 {
-    const long long n_rt = (N + (long long)F_N - 1) / F_N;
-    const long long per = std::max(1LL, tiles * n_rt / (16LL * (sm_count() / 2)));
-    return (int)((n_rt + std::min(per, n_rt) - 1) / std::min(per, n_rt));
+    const long long n_rt = (N + (long long)F_N - 1) / F_N, n_ks = (d + F_KS - 1) / F_KS;
+    const long long pairs = std::max(1, sm_count() / 2);
+    const long long per = std::min(n_rt, std::max(1LL, tiles * n_rt / (16 * pairs)));
+    const long long most = (n_rt + per - 1) / per;
+    long long best = -1;
+    int parts = 1;
+    for (long long p = 1; p <= most; ++p) {
+        const long long units = (tiles * p + pairs - 1) / pairs;        // of the busiest pair
+        const bool reread = std::min((long long)tiles, pairs / p) * 1024 * d > 100000000;
+        const long long cost = (units * n_rt + p - 1) / p * n_ks * (reread ? 21 : 20) +
+                               units * (p > 1 ? 50 : 40);
+        if (best < 0 || cost < best) {
+            best = cost;
+            parts = (int)p;
+        }
+    }
+    return parts;
 }
 
-size_t clip_slot_bytes(int tiles, int N)
+size_t clip_slot_bytes(int tiles, int N, int d)
 {
-    const int parts = clip_parts(tiles, N);
+    const int parts = clip_parts(tiles, N, d);
     return parts > 1 ? (size_t)tiles * parts * 2 * F_VEC * sizeof(double) : 0;
 }
 
@@ -522,7 +543,7 @@ mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
                              const unsigned *xrange, const unsigned *vrange, const uint16_t *xs,
                              unsigned *count, double *slot, cudaStream_t stream)
 {
-    const int tiles = clip_tiles(C), parts = clip_parts(tiles, N);
+    const int tiles = clip_tiles(C), parts = clip_parts(tiles, N, d);
 
     CUtensorMap tmX, tmA;
     memset(&tmX, 0, sizeof(tmX));
@@ -628,8 +649,8 @@ static ClipLayout clip_layout(int C, int N, int d, int n_cand)
     l.planes = l.xs + (size_t)N * d * 4;
     l.vrange = l.planes + (size_t)m_max * d * 4;
     l.slot = up(l.vrange + (size_t)m_max * 4);
-    l.count = l.slot + std::max(chunks > 1 ? clip_slot_bytes(clip_tiles(m_max), N) : 0,
-                                clip_slot_bytes(clip_tiles(last), N));
+    l.count = l.slot + std::max(chunks > 1 ? clip_slot_bytes(clip_tiles(m_max), N, d) : 0,
+                                clip_slot_bytes(clip_tiles(last), N, d));
     l.n_count = 2 * ((chunks - 1) * clip_tiles(m_max) + clip_tiles(last));
     l.bytes = up(l.count + (size_t)l.n_count * 4);
     return l;

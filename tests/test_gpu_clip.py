@@ -33,6 +33,8 @@ def run_both(oracle, X, W, bits, n_cand, mode, groups=1):
     (50, 256, 600, 20), (13, 64, 100, 32), (130, 128, 300, 7), (3, 48, 20, 1), (64, 576, 512, 20),
     # more residual vectors than CTAs that write their planes
     (700, 16, 33, 20),
+    # row tiles in unequal parts (8 in 3, 5 in 2), and whole where there are several
+    (260, 64, 1900, 20), (330, 16, 1100, 20), (640, 16, 600, 20),
     # other rows: fp32 register tiles
     (11, 147, 129, 20), (4, 33, 70, 5), (2, 17, 300, 32),
 ])
