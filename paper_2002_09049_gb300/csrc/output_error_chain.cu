@@ -17,6 +17,8 @@
 // has its own power of two 2^e_n (from its largest magnitude): the chain runs on
 // y_n 2^e_n = y_{n+1} 2^{e_{n+1}} * 2^{e_n - e_{n+1}} + (s_n 2^e_n) P_n, so neither the values nor
 // their squares leave fp32's range before the exact rescaling in double at the end.
+// A scale may be NaN (a refused step of the adaptive grid, with every later one): the chain then starts
+// at the last residual before it, and the errors after it are NaN.
 // Codes that are not nearest values (a caller's own) can make a residual grow; a channel whose
 // largest magnitude more than doubles at a step, or whose scale exceeds four times it, is computed
 // by plain fp32 sums over its residuals instead (slow_channel).
@@ -295,8 +297,10 @@ __device__ __forceinline__ bool is_slow(const unsigned *__restrict__ vrange,
     float vr = __uint_as_float(__ldg(vrange + k * KP1));
 #pragma unroll 1
     for (int n = 0; n < KP1 - 1; ++n) {
+        const float sn = __ldg(scales + k * (KP1 - 1) + n);
+        if (isnan(sn)) break;   // (the chain ends here)
         const float vn = __uint_as_float(__ldg(vrange + k * KP1 + n + 1));
-        slow |= grows(vr, vn, __ldg(scales + k * (KP1 - 1) + n));
+        slow |= grows(vr, vn, sn);
         vr = vn;
     }
     return slow;
@@ -605,8 +609,15 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
 #pragma unroll
                         for (int n = 0; n < K; ++n)
                             sc[i][n] = own ? __ldg(scales + (size_t)(k0 + c) * K + n) : 0.0f;
+                        // points from a NaN scale on are left out of the last residual
+                        int cut = K;
+#pragma unroll
+                        for (int n = K - 1; n >= 0; --n) cut = isnan(sc[i][n]) ? n : cut;
+#pragma unroll
+                        for (int n = 0; n < K; ++n)
+                            if (n >= cut) sc[i][n] = 0.0f;
                         vf[i] = own ? pow2f(f16_scale_exp(__uint_as_float(
-                                          __ldg(vrange + (size_t)(k0 + c) * KP1 + K))))
+                                          __ldg(vrange + (size_t)(k0 + c) * KP1 + cut))))
                                     : 0.0f;
                     }
                 }
@@ -838,17 +849,25 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
         };
         for (int tile = tile0; tile < tile1; ++tile) {
             int me = 0;
-            bool slow = false;
+            bool slow = false, after = false;
             // a new tile: the chain's constants of both CTAs' operand rows, this CTA's slow
             // channels (every warp is done with the last tile's: the barrier at its end)
             float2 cf = make_float2(0.0f, 0.0f);
             const int k = (tile * 2 + (et >> 7)) * CH + mc;
             if (mc < CH && k < C && mn <= K && MPQ_IN((size_t)k * KP1 + mn, (size_t)C * KP1)) {
-                const float vr = __uint_as_float(__ldg(vrange + (size_t)k * KP1 + mn));
+                const float *sk = scales + (size_t)k * K;
+                const unsigned *vk = vrange + (size_t)k * KP1;
+                // the first NaN scale ends the chain: its point and the later ones are no part of
+                // the residual it starts from (the producers'), and the errors after it are NaN
+                int cut = K;
+#pragma unroll
+                for (int n = K - 1; n >= 0; --n) cut = isnan(__ldg(sk + n)) ? n : cut;
+                after = mn > cut;
+                const float vr = __uint_as_float(__ldg(vk + min(mn, cut)));
                 me = f16_scale_exp(vr);
-                if (mn < K) {
-                    const float vn = __uint_as_float(__ldg(vrange + (size_t)k * KP1 + mn + 1));
-                    const float sn = __ldg(scales + (size_t)k * K + mn);
+                if (mn < cut) {
+                    const float vn = __uint_as_float(__ldg(vk + mn + 1));
+                    const float sn = __ldg(sk + mn);
                     const int de = me - f16_scale_exp(vn);
                     // (beyond 2^-126 the later residuals are nothing beside this one; a
                     // growing residual is a slow channel's)
@@ -858,6 +877,8 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                         ctl.slow[mc] = tile + 1;
                         ctl.any_slow = 1;
                     }
+                } else {
+                    cf.x = 1.0f;
                 }
             }
             ctl.coef[et] = cf;
@@ -976,7 +997,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                     MPQ_IN((size_t)k * KP1 + mn, (size_t)C * KP1)) {
                     // exact: undo the operand scales
                     err[(size_t)k * KP1 + mn] =
-                        (float)(s / (double)N * pow2d(-2 * (ctl.xexp + me)));
+                        after ? NAN : (float)(s / (double)N * pow2d(-2 * (ctl.xexp + me)));
                 }
             }
             stop = __any_sync(0xffffffffu, stop || *abort_flag);

@@ -212,3 +212,37 @@ def test_rows_of_any_length(gpu, oracle, C, d, N, K, off):
     torch.cuda.synchronize()
     assert torch.equal(e, e_fixed) and torch.equal(e, e_rmax)
     compare_err(e.cpu().numpy(), oracle.output_error(X, 1, W, o["codes"], o["scales"], K))
+
+
+@pytest.mark.parametrize("C,d,N,K", [(60, 144, 300, 5), (25, 257, 257, 9), (30, 1040, 600, 16), (90, 64, 70, 1)])
+def test_scales_that_end_in_nan(gpu, oracle, C, d, N, K):
+    """A channel whose points end at a NaN scale (a refused step of the adaptive grid: this and every
+    later scale NaN, codes 0) keeps its errors before that point."""
+    W = wlm.random_weights(C, d, 7 * C + d, "normal")
+    q = oracle.quantize_layer(W, 4, 32, K)
+    codes, scales = q["codes"].copy(), q["scales"].copy()
+    for k, n in ((0, 0), (1, K - 1), (C // 2, K // 2), (C - 1, 0)):
+        scales[k, n:] = np.nan
+        codes[n:, k] = 0
+    X = wlm.random_calibration(N, d, 5)
+    e = gpu_err(X, W, codes, scales, K)
+    o = oracle.output_error(X, 1, W, codes, scales, K)
+    assert np.array_equal(np.isnan(e), np.isnan(o)) and np.isnan(o).any()
+    compare_err(np.where(np.isnan(o), 0, e), np.where(np.isnan(o), 0, o))
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(gpu)
+    e_fixed = binding.mpq_output_error_noalloc(t(X), t(W), t(codes), t(scales), K).cpu().numpy()
+    assert np.array_equal(e, e_fixed, equal_nan=True)
+
+
+def test_refused_steps_of_the_adaptive_grid(gpu, oracle):
+    """The adaptive grid's refusals through the output error: errors up to the refused step."""
+    W = wlm.random_weights(64, 144, 11, "normal")
+    X = wlm.random_calibration(300, 144, 12)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(gpu)
+    _, _, _, ncand = binding.mpq_quantize_layer_adaptive(t(W), 4, 4, max_cand=10 ** 15)
+    cap = int(ncand.float().median())   # (about half of the steps refused)
+    codes, scales, _, _ = binding.mpq_quantize_layer_adaptive(t(W), 4, 4, max_cand=cap)
+    e = binding.mpq_output_error(t(X), t(W), codes, scales, 4).cpu().numpy()
+    o = oracle.output_error(X, 1, W, codes.cpu().numpy(), scales.cpu().numpy(), 4)
+    assert np.array_equal(np.isnan(e), np.isnan(o)) and np.isnan(o).any() and np.isfinite(o[:, 0]).all()
+    compare_err(np.where(np.isnan(o), 0, e), np.where(np.isnan(o), 0, o))
