@@ -115,6 +115,12 @@ mpq_status mpq_quantize_layer(const float *W, int C, int d, int bits, int G,
  *   N       calibration rows, >= 1.
  *   groups  1 or C.
  *   W, codes, scales, C, d, k_max   as produced by / passed to mpq_quantize_layer.
+ *           Other codes and scales are taken too.  With groups == 1, channels whose residuals grow (by
+ *           more than a factor of 4^(1/k_max) at a point, which nearest codes never do), whose
+ *           scales exceed four times their residual, or end in NaN (their errors from that point on
+ *           are NaN) are computed apart, with plain fp32 sums: hundreds of microseconds a channel and
+ *           more on long rows, one channel per SM at a time (mpq_output_error_noalloc: two per tile of
+ *           channels).  Not with rmax, whose ranges are those of the search's own codes.
  *   rmax    [C][k_max+1] fp32 or NULL: the rmax output of the mpq_quantize_layer call that made
  *           codes and scales (max |r| of every residual vector).  Given, the tensor-core path's
  *           range pass reads X alone instead of X, W and every code plane; NULL, it measures the

@@ -17,11 +17,14 @@
 // has its own power of two 2^e_n (from its largest magnitude): the chain runs on
 // y_n 2^e_n = y_{n+1} 2^{e_{n+1}} * 2^{e_n - e_{n+1}} + (s_n 2^e_n) P_n, so neither the values nor
 // their squares leave fp32's range before the exact rescaling in double at the end.
-// A scale may be NaN (a refused step of the adaptive grid, with every later one): the chain then starts
-// at the last residual before it, and the errors after it are NaN.
-// Codes that are not nearest values (a caller's own) can make a residual grow; a channel whose
-// largest magnitude more than doubles at a step, or whose scale exceeds four times it, is computed
-// by plain fp32 sums over its residuals instead (slow_channel).
+// Codes that are not nearest values (a caller's own) can make a residual grow, and the chain then ends in
+// differences: where a later residual's largest magnitude is g times an earlier one's, that one's
+// error is g times as far from 64-bit sums (4e-7 g; the contraction of residual vectors: 1.5e-6).  A
+// channel that can reach g = 4, whose scale exceeds four times its residual, or whose scales end in NaN
+// (a refused step of the adaptive grid: the errors before it are wanted) is computed by plain fp32
+// sums over its residuals instead (slow_channels.cuh): by blocks of the pass that splits X, or here
+// with RAWX, which has no such pass.  Where the caller has the ranges from the greedy search, whose
+// codes are nearest values, no channel is looked at.
 //
 // Layout.  Two CTAs on neighbouring SMs (a cluster) issue MMAs of M = 256 calibration rows by
 // N = 256 operand rows: each CTA holds 128 calibration rows (hi and lo tiles) and 128 operand rows
@@ -63,6 +66,7 @@
 
 #include "mpq_internal.cuh"
 #include "pair_common.cuh"
+#include "slow_channels.cuh"
 #include "sm100.cuh"
 #include "tf32_operands.cuh"
 #include "waits.cuh"
@@ -91,10 +95,15 @@ constexpr int E_THREADS = 512;
 // 4.07 and 271, 6 * 256: 4.20 and 209)
 constexpr int E_X_EPI = 4 * 256;
 // registers per thread after setmaxnreg: warpgroups 0-1 and 2-3 (epilogue); together exactly what
-// the launch holds (512 threads x 128)
-constexpr int E_REGS_LOW = 80;
-constexpr int E_REGS_HIGH = 176;
-static_assert(256 * E_REGS_LOW + 256 * E_REGS_HIGH == E_THREADS * 128, "register split");
+// the launch holds (512 threads x 128).  With many points the producers bound a step as much as the
+// MMAs do, and get what the epilogue's sums leave: k_max = 8, 11008 x 4096 2.12 ms with 80 and 176,
+// 2.065 with 96 and 160; 2048 x 2048, N = 1024 k_max = 16 246 and 212 us, k_max = 4 88 and 90.  RAWX
+// has the epilogue split X as well.
+template <int K, bool RAWX>
+struct ERegs {
+    static constexpr int LOW = RAWX || K <= 4 ? 80 : 96, HIGH = 256 - LOW;
+    static_assert(256 * LOW + 256 * HIGH == E_THREADS * 128, "register split");
+};
 constexpr int E_TILE = 128 * 128;          // 16 KB: 128 rows of 128 bytes (128-byte swizzle)
 constexpr int E_XSET = 2 * E_TILE;         // hi and lo tiles of X
 constexpr int E_MAX_STAGES = 3;            // operand-row tiles
@@ -127,7 +136,7 @@ struct ChainCtrl {
     int xexp;
     int last[2];                    // this CTA was the last to leave a tile's sums
     float2 coef[E_N];               // per operand row of the pair: (2^{e_n - e_{n+1}}, s_n 2^e_n)
-    int any_slow;                   // some channel of this CTA is left to slow_channel
+    int any_slow;                   // some channel of this CTA is left to slow_error (RAWX)
     int slow[E_VEC];                // per channel of this CTA: 1 + the last pair tile where it is
     double part[4][E_N];            // per lane quarter: sum over the rows' y^2
     double recv[2][E_VEC];          // the peer's sums for this CTA's channels (alternate tiles)
@@ -282,30 +291,6 @@ __device__ __forceinline__ void chain_x(uint32_t slot, uint32_t xset, int p0, in
     }
 }
 
-// A step where a residual grows as no nearest code makes it (see the top): its largest magnitude
-// before and after, its scale.
-__device__ __forceinline__ bool grows(float vr, float vn, float s)
-{
-    return vn > 2.0f * vr || fabsf(s) > 4.0f * vr;
-}
-
-template <int KP1>
-__device__ __forceinline__ bool is_slow(const unsigned *__restrict__ vrange,
-                                        const float *__restrict__ scales, size_t k)
-{
-    bool slow = false;
-    float vr = __uint_as_float(__ldg(vrange + k * KP1));
-#pragma unroll 1
-    for (int n = 0; n < KP1 - 1; ++n) {
-        const float sn = __ldg(scales + k * (KP1 - 1) + n);
-        if (isnan(sn)) break;   // (the chain ends here)
-        const float vn = __uint_as_float(__ldg(vrange + k * KP1 + n + 1));
-        slow |= grows(vr, vn, sn);
-        vr = vn;
-    }
-    return slow;
-}
-
 // RAWX, rows that a tile copy cannot address: the producer warps and the copy warp each copy a share
 // (part 0 .. E_GATHERERS - 1) of the raw slot of a step (columns x .. x + 63, X rows row0 .. + 127,
 // channels k0 .. + nch - 1), for every row the aligned 16 bytes that hold its 64 elements, and arrive
@@ -383,55 +368,6 @@ __device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane)
     return v[0];
 }
 
-// A channel whose codes are not nearest values: its errors from plain fp32 dot products with its
-// residuals (regenerated 64 elements at a time by the 256 epilogue threads into rsh), 64-element
-// sums added into each row's total, squares compensated.  et: thread 0..255.
-template <int KP1>
-__device__ __noinline__ void slow_channel(const float *__restrict__ X, int N, int d,
-                                          const float *__restrict__ w,
-                                          const int8_t *__restrict__ codes, size_t plane,
-                                          const float *__restrict__ s, int et, float *rsh,
-                                          double *red, float *__restrict__ err)
-{
-    constexpr int K = KP1 - 1;
-    auto sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
-#pragma unroll 1
-    for (int n = 0; n <= K; ++n) {
-        double acc = 0.0;
-#pragma unroll 1
-        for (int t0 = 0; t0 < N; t0 += 256) {
-            const int t = t0 + et;
-            float y = 0.0f;
-#pragma unroll 1
-            for (int j0 = 0; j0 < d; j0 += 64) {
-                sync();   // rsh is no longer read
-                if (et < 64 && j0 + et < d) {
-                    float r = w[j0 + et];
-                    for (int i = 0; i < n; ++i)
-                        r = __fmaf_rn(-s[i], (float)codes[i * plane + j0 + et], r);
-                    rsh[et] = r;
-                }
-                sync();
-                if (t < N) {
-                    float p = 0.0f;
-                    const int jn = min(64, d - j0);
-                    for (int j = 0; j < jn; ++j) p = fmaf(X[(size_t)t * d + j0 + j], rsh[j], p);
-                    y = __fadd_rn(y, p);
-                }
-            }
-            if (t < N) acc += (double)y * (double)y;
-        }
-        red[et] = acc;
-        sync();
-        if (et == 0) {
-            double v = 0.0;
-            for (int i = 0; i < 256; ++i) v += red[i];
-            err[n] = (float)(v / (double)N);
-        }
-        sync();
-    }
-}
-
 // The 256 epilogue threads' barrier, and that of 128 of them (the owners of one CTA's channels).
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void own_sync() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
@@ -445,16 +381,16 @@ struct ChainScratch {
 };
 
 // scales: [C][k_max] point scales; xrange[0], vrange: max|X| and max|r| per residual vector, as
-// float bits; X, W, codes: read only by slow_channel.  tiles: channel tiles of a pair
-// (2 CH channels).  tmX: the split X planes [2][N][d] fp16 (RAWX: X itself), tmW: W, tmQ: the codes.
+// float bits; X, W, codes: read only by gathers and slow_error.  tiles: channel tiles of a pair
+// (2 CH channels).  nearest: every channel's codes are nearest values.  tmX: the split X planes [2][N][d] fp16 (RAWX: X itself), tmW: W, tmQ: the codes.
 template <int KP1, bool RAWX>
 __global__ void __launch_bounds__(E_THREADS, 1)
 output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__ W,
                           const int8_t *__restrict__ codes, const float *__restrict__ scales, int C,
                           int N, int d, const unsigned *__restrict__ xrange,
                           const unsigned *__restrict__ vrange, float *__restrict__ err,
-                          int tiles, int gang, const ChainScratch part, const WaitCtl wc,
-                          const __grid_constant__ CUtensorMap tmX,
+                          int tiles, int gang, bool nearest, const ChainScratch part,
+                          const WaitCtl wc, const __grid_constant__ CUtensorMap tmX,
                           const __grid_constant__ CUtensorMap tmW,
                           const __grid_constant__ CUtensorMap tmQ)
 {
@@ -583,7 +519,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
 
     // one setmaxnreg per warpgroup: 0-1 give registers to 2-3 (epilogue)
     if (warp < E_EPI_WARP0) {
-        setmaxnreg_dec<E_REGS_LOW>();
+        setmaxnreg_dec<ERegs<K, RAWX>::LOW>();
         if (warp < E_PROD_WARPS) {
             // ------------------------------------------------------------ producers
             const int pt = threadIdx.x;
@@ -609,15 +545,8 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
 #pragma unroll
                         for (int n = 0; n < K; ++n)
                             sc[i][n] = own ? __ldg(scales + (size_t)(k0 + c) * K + n) : 0.0f;
-                        // points from a NaN scale on are left out of the last residual
-                        int cut = K;
-#pragma unroll
-                        for (int n = K - 1; n >= 0; --n) cut = isnan(sc[i][n]) ? n : cut;
-#pragma unroll
-                        for (int n = 0; n < K; ++n)
-                            if (n >= cut) sc[i][n] = 0.0f;
                         vf[i] = own ? pow2f(f16_scale_exp(__uint_as_float(
-                                          __ldg(vrange + (size_t)(k0 + c) * KP1 + cut))))
+                                          __ldg(vrange + (size_t)(k0 + c) * KP1 + K))))
                                     : 0.0f;
                     }
                 }
@@ -800,7 +729,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
         }
         __syncwarp();
     } else {
-        setmaxnreg_inc<E_REGS_HIGH>();
+        setmaxnreg_inc<ERegs<K, RAWX>::HIGH>();
         // ---------------------------------------------------------------- epilogue
         // lane quarter q (the TMEM lanes this warp may access) and column half h (that CTA's
         // channels); the running sums of this thread's calibration row stay in registers
@@ -849,36 +778,26 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
         };
         for (int tile = tile0; tile < tile1; ++tile) {
             int me = 0;
-            bool slow = false, after = false;
+            bool slow = false;
             // a new tile: the chain's constants of both CTAs' operand rows, this CTA's slow
             // channels (every warp is done with the last tile's: the barrier at its end)
             float2 cf = make_float2(0.0f, 0.0f);
             const int k = (tile * 2 + (et >> 7)) * CH + mc;
             if (mc < CH && k < C && mn <= K && MPQ_IN((size_t)k * KP1 + mn, (size_t)C * KP1)) {
-                const float *sk = scales + (size_t)k * K;
-                const unsigned *vk = vrange + (size_t)k * KP1;
-                // the first NaN scale ends the chain: its point and the later ones are no part of
-                // the residual it starts from (the producers'), and the errors after it are NaN
-                int cut = K;
-#pragma unroll
-                for (int n = K - 1; n >= 0; --n) cut = isnan(__ldg(sk + n)) ? n : cut;
-                after = mn > cut;
-                const float vr = __uint_as_float(__ldg(vk + min(mn, cut)));
+                const float vr = __uint_as_float(__ldg(vrange + (size_t)k * KP1 + mn));
                 me = f16_scale_exp(vr);
-                if (mn < cut) {
-                    const float vn = __uint_as_float(__ldg(vk + mn + 1));
-                    const float sn = __ldg(sk + mn);
+                if (mn < K) {
+                    const float vn = __uint_as_float(__ldg(vrange + (size_t)k * KP1 + mn + 1));
+                    const float sn = __ldg(scales + (size_t)k * K + mn);
                     const int de = me - f16_scale_exp(vn);
                     // (beyond 2^-126 the later residuals are nothing beside this one; a
                     // growing residual is a slow channel's)
                     cf = make_float2(de < -126 ? 0.0f : pow2f(min(de, 126)),
                                      __fmul_rn(sn, pow2f(me)));
-                    if (mine && grows(vr, vn, sn)) {
+                    if (mine && !nearest && slow_point(vr, vn, sn, growth_limit(K))) {
                         ctl.slow[mc] = tile + 1;
-                        ctl.any_slow = 1;
+                        if constexpr (RAWX) ctl.any_slow = 1;
                     }
-                } else {
-                    cf.x = 1.0f;
                 }
             }
             ctl.coef[et] = cf;
@@ -997,7 +916,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                     MPQ_IN((size_t)k * KP1 + mn, (size_t)C * KP1)) {
                     // exact: undo the operand scales
                     err[(size_t)k * KP1 + mn] =
-                        after ? NAN : (float)(s / (double)N * pow2d(-2 * (ctl.xexp + me)));
+                        (float)(s / (double)N * pow2d(-2 * (ctl.xexp + me)));
                 }
             }
             stop = __any_sync(0xffffffffu, stop || *abort_flag);
@@ -1006,17 +925,17 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
     }
 
     cluster_sync();   // nothing of the pair's is in flight: the peer's sums have been read
-    if (warp >= E_EPI_WARP0 && ctl.any_slow && !*abort_flag) {
-        // slow channels, by the pair that has a tile's first row tile
-        for (int tl = tile0; tl < tile1; ++tl) {
-            if (rt_lo(tl) != 0) continue;
-            for (int c = 0; c < n_chan(tl); ++c) {
-                const size_t k = (size_t)(chan0(tl) + c);
-                if (!is_slow<KP1>(vrange, scales, k)) continue;
-                slow_channel<KP1>(X, N, d, W + k * d, codes + k * d, (size_t)C * d, scales + k * K,
-                                  (int)threadIdx.x - E_EPI_WARP0 * 32,
-                                  reinterpret_cast<float *>(ctl.coef), &ctl.part[0][0],
-                                  err + k * KP1);
+    if constexpr (RAWX) {
+        if (warp >= E_EPI_WARP0 && ctl.any_slow && !*abort_flag) {
+            // slow channels, by the pair that has a tile's first row tile
+            const SlowLayer layer = {X, W, codes, scales, vrange, err, C, N, d, K};
+            for (int tl = tile0; tl < tile1; ++tl) {
+                if (rt_lo(tl) != 0) continue;
+                for (int c = 0; c < n_chan(tl); ++c) {
+                    if (!is_slow(layer, chan0(tl) + c)) continue;
+                    for (int n = warp - E_EPI_WARP0; n <= K; n += S_WARPS)
+                        slow_error(layer, chan0(tl) + c, n, lane);
+                }
             }
         }
     }
@@ -1030,8 +949,8 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
 template <int KP1, bool RAWX>
 mpq_status launch_chain(const float *X, const void *A, int N, const float *W, const int8_t *codes,
                         const float *scales, int C, int d, float *err, const unsigned *xrange,
-                        const unsigned *vrange, const PadRows &pad, void *part, size_t part_bytes,
-                        cudaStream_t stream)
+                        const unsigned *vrange, bool nearest, const PadRows &pad, void *part,
+                        size_t part_bytes, cudaStream_t stream)
 {
     using G = EGeo<KP1, RAWX>;
     const int n_rt = (int)((N + (long long)E_M - 1) / E_M);
@@ -1139,7 +1058,7 @@ mpq_status launch_chain(const float *X, const void *A, int N, const float *W, co
     const mpq_status wst = wait_ctl(&wc);
     if (wst != MPQ_OK) return wst;
     e = cudaLaunchKernelEx(&cfg, output_error_chain_kernel<KP1, RAWX>, X, W, codes, scales, C, N, d,
-                           xrange, vrange, err, tiles, gang, sp, wc, tmX, tmW, tmQ);
+                           xrange, vrange, err, tiles, gang, nearest, sp, wc, tmX, tmW, tmQ);
     return cuda_status(e, "output-error kernel launch");
 }
 
@@ -1163,16 +1082,16 @@ int chain_max_gang(int N) { return N <= E_M ? 1 : E_MAX_GANG; }
 mpq_status launch_output_error_chain(const float *X, int N, const float *W, const int8_t *codes,
                                      const float *scales, int C, int d, int k_max, float *err,
                                      const unsigned *xrange, const unsigned *vrange,
-                                     const uint16_t *xs, const PadRows &pad, void *part,
+                                     bool nearest, const uint16_t *xs, const PadRows &pad, void *part,
                                      size_t part_bytes, cudaStream_t stream)
 {
     switch (k_max) {
 #define MPQ_CASE(n)                                                                               \
     case n:                                                                                       \
         return xs ? launch_chain<n + 1, false>(X, xs, N, W, codes, scales, C, d, err, xrange,     \
-                                               vrange, pad, part, part_bytes, stream)             \
+                                               vrange, nearest, pad, part, part_bytes, stream)    \
                   : launch_chain<n + 1, true>(X, X, N, W, codes, scales, C, d, err, xrange,       \
-                                              vrange, pad, part, part_bytes, stream);
+                                              vrange, nearest, pad, part, part_bytes, stream);
         MPQ_CASE(1) MPQ_CASE(2) MPQ_CASE(3) MPQ_CASE(4) MPQ_CASE(5) MPQ_CASE(6) MPQ_CASE(7)
         MPQ_CASE(8) MPQ_CASE(9) MPQ_CASE(10) MPQ_CASE(11) MPQ_CASE(12) MPQ_CASE(13) MPQ_CASE(14)
         MPQ_CASE(15) MPQ_CASE(16)

@@ -39,6 +39,7 @@
 
 #include "mpq_internal.cuh"
 #include "pair_common.cuh"
+#include "slow_channels.cuh"
 #include "rounding.cuh"
 #include "sm100.cuh"
 #include "tf32_operands.cuh"
@@ -384,16 +385,39 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
     }
 }
 
-// X * 2^e split into fp16 hi and lo planes ([2][N][d]: hi at 0, lo at N d), 8 elements a thread
-// per step, e from max|X| (xrange[0]) as the contraction's operand scale.
-__global__ void __launch_bounds__(256)
+// The slow channels of the output error that this split is for (none for the clipping search), by the
+// blocks from `first` on: a block looks at channels a grid of them apart, a lane each (every warp at
+// all of them: where there are none that is over in a latency or two, before the split is), and its
+// warps take the errors of the slow ones in turn.
+__device__ __forceinline__ void split_slow_channels(const SlowLayer &l, int first)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int step = (int)gridDim.x - first;
+    for (int k0 = (int)blockIdx.x - first; k0 < l.C; k0 += 32 * step) {
+        const long long k = k0 + (long long)lane * step;
+        unsigned slow = __ballot_sync(0xffffffffu, k < l.C && is_slow(l, (int)k));
+        for (; slow; slow &= slow - 1)
+            for (int n = warp; n <= l.K; n += S_WARPS)
+                slow_error(l, k0 + (__ffs(slow) - 1) * step, n, lane);
+    }
+}
+
+// X * 2^e split into fp16 hi and lo planes ([2][N][d]: hi at 0, lo at N d) by the first `blocks` blocks,
+// 8 elements a thread per step, e from max|X| (xrange[0]) as the contraction's operand scale.
+template <bool SLOW>
+__global__ void __launch_bounds__(256, SLOW ? 4 : 1)
 f16_split_kernel(const float4 *__restrict__ X, long long n8, const unsigned *__restrict__ xrange,
-                 uint4 *__restrict__ hi, uint4 *__restrict__ lo)
+                 uint4 *__restrict__ hi, uint4 *__restrict__ lo, int blocks,
+                 const __grid_constant__ SlowLayer slow)
 {
     griddep_launch();
     griddep_wait();
+    if (SLOW && (int)blockIdx.x >= blocks) {
+        split_slow_channels(slow, blocks);
+        return;
+    }
     const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
-    const long long stride = (long long)gridDim.x * blockDim.x;
+    const long long stride = (long long)blocks * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += stride) {
         const float4 a = __ldg(X + 2 * i), b = __ldg(X + 2 * i + 1);
         uint4 H, L;
@@ -407,16 +431,22 @@ f16_split_kernel(const float4 *__restrict__ X, long long n8, const unsigned *__r
 }
 
 // The same for rows of any length and alignment, into rows of dp elements (zeros from d on).
-__global__ void __launch_bounds__(256)
+template <bool SLOW>
+__global__ void __launch_bounds__(256, SLOW ? 4 : 1)
 f16_split_rows_kernel(const float *__restrict__ X, int N, int d, int dp,
                       const unsigned *__restrict__ xrange, uint4 *__restrict__ hi,
-                      uint4 *__restrict__ lo)
+                      uint4 *__restrict__ lo, int blocks,
+                      const __grid_constant__ SlowLayer slow)
 {
     griddep_launch();
     griddep_wait();
+    if (SLOW && (int)blockIdx.x >= blocks) {
+        split_slow_channels(slow, blocks);
+        return;
+    }
     const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
     const int d8 = dp / 8;
-    const long long n8 = (long long)N * d8, stride = (long long)gridDim.x * blockDim.x;
+    const long long n8 = (long long)N * d8, stride = (long long)blocks * blockDim.x;
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long dt = stride / d8;               // rows and items that a stride advances
     const int dj = (int)(stride - dt * d8);
@@ -604,25 +634,26 @@ mpq_status launch_clip_error(const void *A, int N, int C, int d, float *err,
 
 }  // namespace
 
-// X split into the fp16 planes xs ([2][N][dp]) on `stream`.
+// X split into the fp16 planes xs ([2][N][dp]) and the slow channels' errors on `stream`.
 cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange, uint16_t *xs,
-                           cudaStream_t stream)
+                           const SlowLayer &slow, cudaStream_t stream)
 {
     const int dp = (d + 15) / 16 * 16;
     const long long n8 = (long long)N * dp / 8;
-    const int sb = (int)std::min<long long>((n8 + 255) / 256, 4LL * sm_count());
+    const int sb = (int)std::max(1LL, std::min<long long>((n8 + 255) / 256, 4LL * sm_count()));
     cudaLaunchAttribute attr[1] = {after_previous_kernel()};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::max(sb, 1), 1, 1);
+    cfg.gridDim = dim3((unsigned)(sb + std::min(slow.C, sm_count())), 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     uint4 *hi = reinterpret_cast<uint4 *>(xs), *lo = reinterpret_cast<uint4 *>(xs + (size_t)N * dp);
     if (d != dp || ((uintptr_t)X & 15) != 0)
-        return cudaLaunchKernelEx(&cfg, f16_split_rows_kernel, X, N, d, dp, xrange, hi, lo);
-    return cudaLaunchKernelEx(&cfg, f16_split_kernel, reinterpret_cast<const float4 *>(X), n8, xrange,
-                              hi, lo);
+        return cudaLaunchKernelEx(&cfg, slow.C ? f16_split_rows_kernel<true> : f16_split_rows_kernel<false>,
+                                  X, N, d, dp, xrange, hi, lo, sb, slow);
+    return cudaLaunchKernelEx(&cfg, slow.C ? f16_split_kernel<true> : f16_split_kernel<false>,
+                              reinterpret_cast<const float4 *>(X), n8, xrange, hi, lo, sb, slow);
 }
 
 // Channels per chunk of residual planes: whole channels, at most 4 GiB of planes at a time.
@@ -676,7 +707,7 @@ mpq_status launch_clip_f16(const float *X, int N, const float *W, const float *c
     unsigned *count = reinterpret_cast<unsigned *>(p + l.count);
     mpq_status st = launch_x_range(X, N, d, xrange, count, l.n_count, stream);
     if (st != MPQ_OK) return st;
-    cudaError_t e = launch_x_split(X, N, d, xrange, xs, stream);
+    cudaError_t e = launch_x_split(X, N, d, xrange, xs, SlowLayer{}, stream);
     if (e != cudaSuccess) return cuda_status(e, "X split kernel launch");
     for (int c0 = 0; c0 < C && st == MPQ_OK; c0 += cc) {
         const int cn = std::min(cc, C - c0);

@@ -20,6 +20,7 @@
 
 #include "mpq_internal.cuh"
 #include "pair_common.cuh"
+#include "slow_channels.cuh"
 #include "sm100.cuh"
 
 MPQ_CHECKED_UNIT("output_error_pair.cu");
@@ -220,13 +221,14 @@ mpq_status launch_pair(const float *X, int N, const float *W, const int8_t *code
         launch_ranges<KP1>(X, N, W, codes, scales, C, d, rmax == nullptr, range,
                            reinterpret_cast<unsigned *>(part), 2 * tiles, pad, stream),
         "output-error range pre-pass");
-    if (r == MPQ_OK && xs)
-        r = cuda_status(launch_x_split(X, N, d, range, xs, stream), "X split kernel launch");
-    if (r == MPQ_OK) {
-        const unsigned *vr = rmax ? reinterpret_cast<const unsigned *>(rmax) : range + 1;
-        r = launch_output_error_chain(X, N, W, codes, scales, C, d, KP1 - 1, err, range, vr, xs,
-                                      pad, part, part_bytes, stream);
+    const unsigned *vr = rmax ? reinterpret_cast<const unsigned *>(rmax) : range + 1;
+    if (r == MPQ_OK && xs) {
+        const SlowLayer slow = {X, W, codes, scales, vr, err, rmax ? 0 : C, N, d, KP1 - 1};
+        r = cuda_status(launch_x_split(X, N, d, range, xs, slow, stream), "X split kernel launch");
     }
+    if (r == MPQ_OK)
+        r = launch_output_error_chain(X, N, W, codes, scales, C, d, KP1 - 1, err, range, vr,
+                                      rmax != nullptr, xs, pad, part, part_bytes, stream);
     if (!ext_range) {
         const cudaError_t ef = cudaFreeAsync(range, stream);
         if (r == MPQ_OK) r = cuda_status(ef, "scratch release (cudaFreeAsync)");

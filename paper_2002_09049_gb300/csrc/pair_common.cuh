@@ -78,12 +78,15 @@ mpq_status launch_x_range(const float *X, int N, int d, unsigned *range, unsigne
                           int n_count, cudaStream_t stream);
 
 // Host: X * 2^e (e from xrange[0]) split into the fp16 hi and lo planes xs ([2][N][dp], dp = d
-// rounded up to 16, the rest of a row zero).
+// rounded up to 16, the rest of a row zero), and the errors of a layer's slow channels
+// (slow_channels.cuh; C = 0: none).
+struct SlowLayer;
 cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange, uint16_t *xs,
-                           cudaStream_t stream);
+                           const SlowLayer &slow, cudaStream_t stream);
 
 // Host: the output error of the greedy points (output_error_chain.cu), with its ranges ready on
-// `stream` (xrange[0] = max|X|, vrange = max|r| per residual vector, float bits); xs: the split X
+// `stream` (xrange[0] = max|X|, vrange = max|r| per residual vector, float bits); nearest: the codes are
+// nearest values (else slow channels are left out, or with xs NULL computed here); xs: the split X
 // planes, or NULL (the contraction then splits X itself); pad: padded copies of W and the codes,
 // or none (with xs, W and codes are then rows a tile copy can address); part: part_bytes of 256-byte aligned
 // scratch for partial sums, at least chain_count_bytes(tiles) and that much of it zeroed on
@@ -91,7 +94,7 @@ cudaError_t launch_x_split(const float *X, int N, int d, const unsigned *xrange,
 mpq_status launch_output_error_chain(const float *X, int N, const float *W, const int8_t *codes,
                                      const float *scales, int C, int d, int k_max, float *err,
                                      const unsigned *xrange, const unsigned *vrange,
-                                     const uint16_t *xs, const PadRows &pad, void *part,
+                                     bool nearest, const uint16_t *xs, const PadRows &pad, void *part,
                                      size_t part_bytes, cudaStream_t stream);
 int chain_tiles(int C, int k_max);   // channel tiles of a CTA pair
 size_t chain_count_bytes(int tiles);

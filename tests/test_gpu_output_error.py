@@ -181,6 +181,40 @@ def test_codes_that_are_not_nearest_values(gpu, oracle, K):
     compare_err(gpu_err(X, W, codes, scales, K), oracle.output_error(X, 1, W, codes, scales, K))
 
 
+@pytest.mark.parametrize("grow", [1.15, 1.35, 1.9])
+def test_residuals_that_grow_step_by_step(gpu, oracle, grow):
+    """Codes that add to the residual, a little at each of 16 points (9, 122 and 29,000 times in all):
+    no single step doubles it, and the first errors are as exact as the last."""
+    C, d, N, K = 20, 160, 300, 16
+    W = wlm.random_weights(C, d, 3, "normal")
+    codes, scales = np.zeros((K, C, d), np.int8), np.zeros((C, K), np.float32)
+    r = W.copy()
+    for n in range(K):
+        scales[:, n] = np.abs(r).max(1) * np.float32(grow - 1) / 7
+        codes[n] = np.rint(-r * np.float32(grow - 1) / scales[:, n:n + 1]).clip(-7, 7)
+        r = r - scales[:, n:n + 1] * codes[n]
+    X = wlm.random_calibration(N, d, 5)
+    compare_err(gpu_err(X, W, codes, scales, K), oracle.output_error(X, 1, W, codes, scales, K))
+
+
+@pytest.mark.parametrize("C,d,N,K", [(60, 144, 300, 5), (400, 64, 70, 1), (25, 257, 257, 9),
+                                     (30, 1040, 33, 16), (15, 601, 100, 16), (9, 8192, 40, 8)])
+def test_every_channel_grows(gpu, oracle, C, d, N, K):
+    """Layers of channels that the chain cannot take, more of them than blocks that look for them, rows
+    longer than shared memory holds residuals of: the pooled and the fixed-scratch entry points (which
+    regenerate different lengths at a time) give the same errors bit for bit."""
+    rng = np.random.default_rng(C + d)
+    W = wlm.random_weights(C, d, 21, "normal")
+    codes = rng.integers(-7, 8, size=(K, C, d)).astype(np.int8)
+    scales = rng.uniform(1, 3, size=(C, K)).astype(np.float32)
+    X = wlm.random_calibration(N, d, 5)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(gpu)
+    args = (t(X), t(W), t(codes), t(scales), K)
+    e = binding.mpq_output_error(*args)
+    assert torch.equal(e, binding.mpq_output_error_noalloc(*args))
+    compare_err(e.cpu().numpy(), oracle.output_error(X, 1, W, codes, scales, K))
+
+
 # rows that tile copies cannot address: around 16 elements and a 64-element step, channel and row
 # tile edges as above, where the chain takes them and just below; off: elements that X, W and
 # (x 4) the codes start past a 16-byte boundary
