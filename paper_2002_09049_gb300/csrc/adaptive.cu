@@ -1249,8 +1249,8 @@ mpq_status launch_adaptive(const float *W, int C, int d, int qmax, int k_max, do
     const int cap = (int)(ev > d ? ev : d);
     const int grid = (int)std::min<long long>(C, (long long)sm_count() * A_CTAS_PER_SM);
     const size_t smem = adaptive_smem(d);
-    cudaError_t e = cudaFuncSetAttribute(adaptive_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    static std::atomic<int> limit[kMaxDevices];
+    cudaError_t e = allow_smem(reinterpret_cast<const void *>(adaptive_kernel), limit, smem);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute (adaptive grid)");
     uint2 *scratch = nullptr;
     const mpq_status st = pool_scratch(reinterpret_cast<void **>(&scratch),

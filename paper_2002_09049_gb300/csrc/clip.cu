@@ -474,12 +474,13 @@ mpq_status launch_clip(const float *X, int N, int groups, const float *W, int C,
                                    (const float *)clip, err);
         } else {
             const size_t smem = (size_t)CL_CHUNK * d * sizeof(float);
-            if ((long long)smem > max_smem_optin()) {
+            constexpr int fixed = CL_THREADS / 32 * CL_CHUNK * (int)sizeof(float);
+            if ((long long)smem > max_smem_optin() - fixed) {
                 set_error("clip search with d = %d needs %zu bytes of shared memory", d, smem);
                 return MPQ_ERR_UNSUPPORTED;
             }
-            e = cudaFuncSetAttribute(clip_errors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
+            static std::atomic<int> limit[kMaxDevices];
+            e = allow_smem(reinterpret_cast<const void *>(clip_errors_kernel), limit, smem);
             if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
             const dim3 grid((unsigned)C, (unsigned)((n_cand + CL_CHUNK - 1) / CL_CHUNK));
             clip_errors_kernel<<<grid, CL_THREADS, smem, stream>>>(X, N, W, C, d, qmax, n_cand, clip,

@@ -271,8 +271,9 @@ mpq_status launch_grouped(const float *X, int N, const float *W, const int8_t *c
                   KP1 - 1, smem);
         return MPQ_ERR_UNSUPPORTED;
     }
-    cudaError_t e = cudaFuncSetAttribute(output_error_grouped_kernel<KP1>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<int> limit[kMaxDevices];
+    cudaError_t e = allow_smem(reinterpret_cast<const void *>(output_error_grouped_kernel<KP1>), limit,
+                               smem);
     if (e == cudaSuccess) {
         output_error_grouped_kernel<KP1><<<C, GR_THREADS, smem, stream>>>(X, N, W, codes, scales,
                                                                           C, d, err);

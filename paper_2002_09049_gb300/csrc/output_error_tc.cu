@@ -420,8 +420,9 @@ mpq_status launch_tc(const float *X, int N, const float *W, const int8_t *codes,
     const bool vec_ok = (d % 4 == 0) && ((uintptr_t)X % 16 == 0) && ((uintptr_t)W % 16 == 0) &&
                         ((uintptr_t)codes % 4 == 0);
 
-    cudaError_t e = cudaFuncSetAttribute(output_error_tc_kernel<KP1>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    static std::atomic<int> limit[kMaxDevices];
+    cudaError_t e = allow_smem(reinterpret_cast<const void *>(output_error_tc_kernel<KP1>), limit,
+                               TC_SMEM);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute");
 
     cudaLaunchConfig_t cfg = {};
