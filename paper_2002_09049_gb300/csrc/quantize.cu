@@ -619,7 +619,8 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
             // candidate scales s_g = fl(f_g * smax) exactly as defined; fl(1/f_g) * fl(1/smax)
             // is within 2^-22 of 1/s_g, which the fast decisions' 2^-20 margin absorbs
             const float smax = __fdiv_rn(m, qmaxf);
-            const float ism = __frcp_rn(smax);
+            // (the fast codes' bound holds for normal reciprocals; a NaN or infinite one takes the division)
+            const float ism = smax < 0x1p120f ? __frcp_rn(smax) : NAN;
             int e;
             frexpf(m, &e);                      // m < 2^e
             // fixed point R = |r| 2^S: on the lattice, exact for every |r| that can reach bucket 1
@@ -1025,6 +1026,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
             if (g < 0 || g >= G) g = G - 1;   // unreachable: every D is finite
             s_best = __fmul_rn(fg(g), smax);
             inv_best = zero_scale ? 0.0f : fi(g) * ism;
+            if (!(inv_best < 0x1p120f)) inv_best = 0.0f;   // (below 2^-120: smax is above 2^120)
         }
 
         // residual update (Eq. 7) and code emission; also the next step's max |r|

@@ -176,3 +176,22 @@ def test_nullable_outputs_and_stream(gpu):
     c2, s2, _, _ = binding.mpq_quantize_layer(W, 4, 32, 3)
     torch.cuda.synchronize()
     assert torch.equal(c1, c2) and torch.equal(s1, s2)
+
+
+@pytest.mark.parametrize("lo,hi", [(-146, -137), (-138, -118), (118, 125)])
+@pytest.mark.parametrize("grid", ["linear", "geometric"])
+def test_codes_where_reciprocals_end(gpu, grid, lo, hi):
+    """Scales whose reciprocals are not normal numbers: the codes are still the division's (Eq. 8)."""
+    G, k_max, d, qmax = 64, 2, 1200, 7
+    rng = np.random.default_rng(hi + 300)
+    W = np.ldexp(rng.uniform(-1, 1, (60, d)), rng.integers(lo, hi, (60, 1))).astype(np.float32)
+    frac = None if grid == "linear" else [16.0 ** ((g + 1 - G) / G) for g in range(G)]
+    codes, scales, _, _ = binding.mpq_quantize_layer(torch.from_numpy(W).to(gpu), 4, G, k_max,
+                                                     grid_frac=frac)
+    codes, scales, r = codes.cpu().numpy(), scales.cpu().numpy(), W
+    for i in range(k_max):
+        s = scales[:, i:i + 1]
+        with np.errstate(divide="ignore", invalid="ignore", over="ignore"):
+            q = np.where(s > 0, np.clip(np.rint(r / s), -qmax, qmax), 0)
+        assert np.array_equal(codes[i], q.astype(np.int8))
+        r = (r.astype(np.float64) - s.astype(np.float64) * q).astype(np.float32)
