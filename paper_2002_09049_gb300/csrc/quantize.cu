@@ -928,7 +928,8 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                 // and the double rate bounds them (6168 x 219, 3 bits, G = 256: 124 us, screened
                 // 97, and 78 with the scans as they are): each warp keeps the candidates whose error interval can contain its own
                 // minimum, D / 2^2e = s'(s'N - 2P') in fp32 with s' = s / 2^e and P' = P 2^-S / 2^e
-                // (both O(1); at most ~8 roundings of 2^-24, the bound allows 2^-20).
+                // (both O(1); at most ~8 roundings of 2^-24, the bound allows 2^-20).  Not where scales
+                // are subnormal: s' is not rounded as they are.
                 float upper = FLT_MAX, pscale = 0.0f, smax_e = 0.0f;
                 auto screened = [&](int g, float &err) {
                     const float sh = fg(g) * smax_e;
@@ -937,7 +938,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                     err = sh * (sh * Nf + 2.0f * Pf) * MPQ_FAST_REL;
                     return sh * (sh * Nf - 2.0f * Pf);
                 };
-                const bool screen = WPC <= 2 && G >= 4 * NT;
+                const bool screen = WPC <= 2 && G >= 4 * NT && __fmul_rn(fg(0), smax) >= FLT_MIN;
                 if (screen) {
                     pscale = ldexpf(1.0f, -S - e);
                     smax_e = ldexpf(smax, -e);

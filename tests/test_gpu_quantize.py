@@ -195,3 +195,20 @@ def test_codes_where_reciprocals_end(gpu, grid, lo, hi):
             q = np.where(s > 0, np.clip(np.rint(r / s), -qmax, qmax), 0)
         assert np.array_equal(codes[i], q.astype(np.int8))
         r = (r.astype(np.float64) - s.astype(np.float64) * q).astype(np.float32)
+
+
+@pytest.mark.parametrize("bits,grid", [(3, "geometric"), (4, "linear"), (4, "geometric"),
+                                       (5, "geometric")])
+def test_subnormal_scales_in_large_layers(gpu, bits, grid):
+    """Channels whose scales are subnormal get the same points in a layer of thousands of channels as
+    in small ones (there: more warps a channel, and no fp32 screen, which does not see how such scales
+    round)."""
+    G, d = 128, 600
+    rng = np.random.default_rng(9)
+    W = np.ldexp(rng.standard_normal((5000, d)), rng.integers(-145, -137, (5000, 1))).astype(np.float32)
+    frac = None if grid == "linear" else [16.0 ** ((g + 1 - G) / G) for g in range(G)]
+    W = torch.from_numpy(W).to(gpu)
+    codes, scales, _, _ = binding.mpq_quantize_layer(W, bits, G, 1, grid_frac=frac)
+    for c in range(0, 2000, 200):
+        q, s, _, _ = binding.mpq_quantize_layer(W[c:c + 200], bits, G, 1, grid_frac=frac)
+        assert torch.equal(s, scales[c:c + 200]) and torch.equal(q, codes[:, c:c + 200])
