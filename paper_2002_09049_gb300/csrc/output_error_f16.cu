@@ -500,7 +500,9 @@ clip_planes_kernel(const float *__restrict__ W, int d, const float *__restrict__
         const long long k = c0 + v / n_cand;
         // clip row of channel k, candidate v mod n_cand: index c0 n_cand + v
         const float sv = __fdiv_rn(__ldg(clip + (long long)c0 * n_cand + v), qmaxf);
-        const float inv = sv > 0.0f ? __frcp_rn(sv) : 0.0f;
+        // (the fast codes' bound holds for normal reciprocals: other scales take the division)
+        const bool normal = sv > 0x1p-120f && sv < 0x1p120f;
+        const float inv = normal ? __frcp_rn(sv) : 0.0f;
         const float m = __ldg(chmax + k);
         const float bound = fmaxf(fminf(m, __fmul_rn(0.5f, sv)), __fmaf_rn(-qmaxf, sv, m));
         const float vf = pow2f(f16_scale_exp(bound));
@@ -511,7 +513,7 @@ clip_planes_kernel(const float *__restrict__ W, int d, const float *__restrict__
             const float4 a = __ldg(w4 + 2 * j), b = __ldg(w4 + 2 * j + 1);
             const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
             float q[8];
-            bool unsure = false;
+            bool unsure = !normal;
 #pragma unroll
             for (int e = 0; e < 8; ++e) q[e] = code_signed_fast(w[e], inv, qmaxf, qlim, tband, unsure);
             if (unsure) {

@@ -164,3 +164,21 @@ def test_planes_in_chunks(gpu, oracle):
         compare_err(err[c0:c0 + 4], o_err[c0:c0 + 4])
     assert np.array_equal(best, oracle.clip_select(err, binding.MPQ_CLIP_PER_CHANNEL))
 
+
+@pytest.mark.parametrize("d,lo,hi", [(64, -146, -130), (64, -131, -118), (64, 118, 124), (50, -146, -130)])
+def test_codes_where_reciprocals_end(gpu, oracle, d, lo, hi):
+    """Scales whose reciprocals are not normal numbers.  A calibration row per element reads the
+    residuals back: err N is the sum of their squares, and each is r = w - s q with the division's q."""
+    rng = np.random.default_rng(d + hi + 300)
+    C, n_cand, bits = 9, 6, 4
+    W = np.ldexp(rng.uniform(-1, 1, (C, d)), rng.integers(lo, hi, (C, 1))).astype(np.float32)
+    big = np.float32(2.0 ** (100 if hi < 0 else -100))       # (errors in fp32's range)
+    X = (np.eye(d) * big).astype(np.float32)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(gpu)
+    clip, err, _ = binding.mpq_clip_search(t(X), t(W), bits, n_cand)
+    clip = clip.cpu().numpy()
+    s = (clip / np.float32(7))[:, :, None]
+    with np.errstate(divide="ignore", invalid="ignore", over="ignore"):
+        q = np.where(s > 0, np.clip(np.rint(W[:, None] / s), -7, 7), 0)
+    r = W[:, None].astype(np.float64) - s.astype(np.float64) * q
+    compare_err(err.cpu().numpy(), ((r.astype(np.float32).astype(np.float64) * big) ** 2).sum(2) / d)
