@@ -815,7 +815,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                                 event_level(a, L, (unsigned int)R,
                                             (unsigned int)((unsigned long long)R >> 32), a * g_per_a);
                         }
-                    } else {   // the queue overflowed (never seen): every such element again
+                    } else {   // the queue overflowed (rows of thousands on the longest lattices): every such element again
                         if constexpr (TM) {
                             for (int cc = 0; cc < tcg; cc += 4) {
                                 float v4[4];
@@ -1308,10 +1308,12 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
     // Warps per channel.  A step's fixed work (scans, fold, decision, barriers) grows with the warps
     // of a channel, so no more of them than leave every channel resident at once, 32 warps an SM
     // (1280 x 320: 2 warps 55 us, 4 warps 82; 1500 x 128, G = 100: 1 warp 47, 2 warps 38), at least ~16 elements per warp (candidates, on rows evaluated
-    // directly), at least 4 warps for rows of 1,024 and more (4096 x 1024, G = 256: 200 us against
-    // 323 with 2), and enough warps per SM (24) for the shared memory the channels need -- on
-    // layers with thousands of long channels, 4-warp groups (more channels per SM, barriers over
-    // fewer warps) measured faster than 8-warp ones (11008 x 4096: 1.51 ms against 1.94).
+    // directly), at least 4 warps for rows of 1,024 and more where the lattice has 500 positions to
+    // scan or the row 2,500 elements, and enough warps per SM (26) for the shared memory the channels
+    // need.  us with 1 / 2 / 4 / 8 warps, 3 points, 4 bits: 3200 x 1500, G = 256 (1,261 positions) 190 / 142 /
+    // 121 / 163, G = 64 (315) 105 / 81 / 92 / 135; 9000 x 1024, G = 32 (158) 110 / 133 / 189 / 300; 4096 x 4096,
+    // G = 32 417 / 252 / 187 / 230.  On 11008 x 4096, 4 warps 1.51 ms, 8 warps 1.94 (before the scans over
+    // odd blocks: 1.30 now).
     const long long warps_gpu = (long long)sm_count() * 32;
     int wpc_c = 1;
     // The event form's step is its elements', which more warps share: as many as fill the GPU, at
@@ -1327,8 +1329,8 @@ mpq_status launch_grid(const float *W, int C, int d, int qmax, int G, const Grid
     else
         while (wpc_e < 8 && wpc_e * 16 <= d) wpc_e *= 2;
     const long long groups_per_sm = (long long)(227 * 1024) / (long long)(per_group + 256);
-    int wpc_s = d >= 1024 && !event ? 4 : 1;
-    while (wpc_s < 8 && groups_per_sm * wpc_s < 24) wpc_s *= 2;
+    int wpc_s = d >= 1024 && !event && (nc >= 500 || d >= 2500) ? 4 : 1;
+    while (wpc_s < 8 && groups_per_sm * wpc_s < (event ? 24 : 26)) wpc_s *= 2;
     int wpc = wpc_c < wpc_e ? wpc_c : wpc_e;
     if (wpc < wpc_s) wpc = wpc_s;
     for (; wpc <= 8; wpc *= 2) {
