@@ -39,6 +39,7 @@ KERNEL_SOURCES = {
                      "paper_2002_09049_gb300/csrc/output_error_pair.cu",
                      "paper_2002_09049_gb300/csrc/pair_common.cuh",
                      "paper_2002_09049_gb300/csrc/output_error_tc.cu",
+                     "paper_2002_09049_gb300/csrc/slow_channels.cuh",
                      "paper_2002_09049_gb300/csrc/sm100.cuh",
                      "paper_2002_09049_gb300/csrc/tf32_operands.cuh",
                      "paper_2002_09049_gb300/csrc/waits.cuh"),
@@ -481,7 +482,8 @@ def dominant_roofline(dominant, fam_ms, fam_work, peaks, peak_src, wl, args, sm_
         return {"kernel": "output_error_chain_kernel (Eq. 11, tcgen05 cta_group::2 kind::f16: the "
                           "points' codes and the last residual's hi/lo halves against X's, 2 (k_max "
                           "+ 2) row passes; after pair_range_kernel and f16_split_kernel; "
-                          "output_error_tc_kernel for rows not 16-byte multiples)",
+                          "output_error_tc_kernel for short or few rows that are not whole "
+                          "aligned 16 bytes)",
                 "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "traffic": traffic,
                 "peak_source": f"{peak_src} bf16 dense burst (the fp16 rate of kind::f16)"}

@@ -8,10 +8,9 @@
 // Three steps, all on the device:
 //   1. candidates: one warp per channel takes max|w| (NaN if a weight is non-finite); per-layer
 //      sets reduce the channels' maxima in one CTA;
-//   2. errors: the CTA-pair tensor-core contraction with residuals generated from W and the
-//      candidate scales on chip (output_error_f16.cu: fp16 hi/lo operands, each residual vector
-//      scaled by a power of two from the bound max(min(max|w|, s/2), max|w| - Qmax s) on its
-//      elements), or,
+//   2. errors: the CTA-pair tensor-core contraction over the candidates' residuals, written once as
+//      fp16 hi/lo planes (output_error_f16.cu; each residual vector scaled by a power of two from
+//      the bound max(min(max|w|, s/2), max|w| - Qmax s) on its elements), or,
 //      for shared inputs whose rows are not 16-byte multiples, register tiles of 64 residual
 //      vectors by 128 calibration rows in fp32 (clip_rows_kernel), or, for per-channel inputs, one
 //      CTA per channel and candidate chunk with the residuals in shared memory and threads over

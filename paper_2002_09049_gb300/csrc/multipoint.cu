@@ -14,8 +14,9 @@
 // into 128-byte-swizzled K-major tiles) against the input rows (int8 by TMA into a raw ring, turned
 // into bf16 exactly by eight producer warps through the fp32 exponent bias).  Products are exact
 // and every partial sum is an integer of magnitude below 2^24 when d * Qmax * 128 < 2^24, so the
-// fp32 accumulator holds the exact dot products (checked on the host; other layers take the
-// integer arithmetic of multipoint_mma_kernel).  A unit of work is two 128-row tiles against 256
+// fp32 accumulator holds the exact dot products (checked on the host; other layers take
+// multipoint_mma_kernel, whose warps each accumulate an eighth of a row exactly in fp32 and add the
+// parts as integers).  A unit of work is two 128-row tiles against 256
 // inputs, K chunks of 64, by a CTA pair (cta_group::2: each CTA holds one row tile and half of the
 // inputs, and gets its row tile's outputs for all of them); resident pairs take units a grid apart
 // (inputs fastest, so the pairs that share row tiles run together and read their codes from L2).

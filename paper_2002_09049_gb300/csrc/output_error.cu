@@ -3,11 +3,13 @@
 // with the residuals r_{k,n+1} regenerated on chip from W, codes and scales by the recursion of
 // Eq. 7 (never materialised in global memory).
 //
-// Shared input (groups = 1) is a dense contraction and runs on the tensor cores: the CTA-pair kernel
-// (output_error_pair.cu) when rows are 16-byte multiples, else the single-CTA one
-// (output_error_tc.cu).  Per-channel input (groups = C, depthwise convolution, d = 9): one CTA per
-// channel, its k_max+1 residuals in shared memory, the channel's own rows of X staged through
-// shared memory with coalesced reads (each read once), threads over the rows.
+// Shared input (groups = 1) is a dense contraction and runs on the tensor cores: the CTA pairs of
+// output_error_chain.cu (through output_error_pair.cu) where rows are whole aligned 16 bytes
+// (tile_rows_ok) or long and many enough for padded copies (output_error_rows_ok), else, and where
+// the pool has no room for those copies, the single-CTA kernel (output_error_tc.cu).  Per-channel
+// input (groups = C, depthwise convolution, d = 9): one CTA per channel, its k_max+1 residuals in
+// shared memory, the channel's own rows of X staged through shared memory with coalesced reads
+// (each read once), threads over the rows; rows of up to 32 elements two a thread.
 #include <math.h>
 
 #include <algorithm>

@@ -815,7 +815,7 @@ quantize_kernel(const float *__restrict__ W, int C, int d, int qmax, int G, cons
                                 event_level(a, L, (unsigned int)R,
                                             (unsigned int)((unsigned long long)R >> 32), a * g_per_a);
                         }
-                    } else {   // the queue overflowed (rows of thousands on the longest lattices): every such element again
+                    } else {   // the queue overflowed (weights that sit on the lattice, such as integers): every such element again
                         if constexpr (TM) {
                             for (int cc = 0; cc < tcg; cc += 4) {
                                 float v4[4];

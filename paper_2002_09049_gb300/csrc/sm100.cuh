@@ -345,8 +345,6 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
            | ((uint32_t)(M >> 4) << 24);  // M / 16
 }
 
-// ---- TMA (bulk tensor copies global -> shared, completion counted on an mbarrier) ------------
-// Arms `bar` for `bytes` of incoming transactions and arrives once.
 // Programmatic dependent launch: griddep_launch lets the next kernel of the stream, if it was launched
 // for it, take SMs as they fall free; its griddep_wait returns once the kernels before it have
 // completed and what they wrote is visible (at once in a kernel launched the ordinary way).
@@ -398,6 +396,8 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+// ---- TMA (bulk tensor copies global -> shared, completion counted on an mbarrier) ------------
+// Arms `bar` for `bytes` of incoming transactions and arrives once.
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
