@@ -477,7 +477,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
         tc_fence_before();
     }
     griddep_wait();                     // nothing above reads global memory
-    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
+    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(ld_after_wait(xrange)));
     cluster_sync();                     // barriers of both CTAs initialised, TMEM allocated
     tc_fence_after();
     const uint32_t tmem = ctl.tmem_base;
@@ -546,7 +546,7 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
                         for (int n = 0; n < K; ++n)
                             sc[i][n] = own ? __ldg(scales + (size_t)(k0 + c) * K + n) : 0.0f;
                         vf[i] = own ? pow2f(f16_scale_exp(__uint_as_float(
-                                          __ldg(vrange + (size_t)(k0 + c) * KP1 + K))))
+                                          ld_after_wait(vrange + (size_t)(k0 + c) * KP1 + K))))
                                     : 0.0f;
                     }
                 }
@@ -784,10 +784,10 @@ output_error_chain_kernel(const float *__restrict__ X, const float *__restrict__
             float2 cf = make_float2(0.0f, 0.0f);
             const int k = (tile * 2 + (et >> 7)) * CH + mc;
             if (mc < CH && k < C && mn <= K && MPQ_IN((size_t)k * KP1 + mn, (size_t)C * KP1)) {
-                const float vr = __uint_as_float(__ldg(vrange + (size_t)k * KP1 + mn));
+                const float vr = __uint_as_float(ld_after_wait(vrange + (size_t)k * KP1 + mn));
                 me = f16_scale_exp(vr);
                 if (mn < K) {
-                    const float vn = __uint_as_float(__ldg(vrange + (size_t)k * KP1 + mn + 1));
+                    const float vn = __uint_as_float(ld_after_wait(vrange + (size_t)k * KP1 + mn + 1));
                     const float sn = __ldg(scales + (size_t)k * K + mn);
                     const int de = me - f16_scale_exp(vn);
                     // (beyond 2^-126 the later residuals are nothing beside this one; a

@@ -152,7 +152,7 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
         tc_fence_before();
     }
     griddep_wait();                     // nothing above reads global memory
-    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(__ldg(xrange)));
+    if (threadIdx.x == 0) ctl.xexp = f16_scale_exp(__uint_as_float(ld_after_wait(xrange)));
     cluster_sync();                     // barriers of both CTAs initialised, TMEM allocated
     tc_fence_after();
     const uint32_t tmem = ctl.tmem_base;
@@ -365,7 +365,7 @@ clip_error_kernel(int C, int N, int d, const unsigned *__restrict__ xrange,
                 const int v = vec0(u) + m;
                 if (write && v < C && MPQ_IN(v, C)) {
                     // exact: undo the operand scales
-                    const int e = ctl.xexp + f16_scale_exp(__uint_as_float(__ldg(vrange + v)));
+                    const int e = ctl.xexp + f16_scale_exp(__uint_as_float(ld_after_wait(vrange + v)));
                     err[v] = (float)(s / (double)N * pow2d(-2 * e));
                 }
             }
@@ -416,7 +416,7 @@ f16_split_kernel(const float4 *__restrict__ X, long long n8, const unsigned *__r
         split_slow_channels(slow, blocks);
         return;
     }
-    const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
+    const float xs = pow2f(f16_scale_exp(__uint_as_float(ld_after_wait(xrange))));
     const long long stride = (long long)blocks * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += stride) {
         const float4 a = __ldg(X + 2 * i), b = __ldg(X + 2 * i + 1);
@@ -444,7 +444,7 @@ f16_split_rows_kernel(const float *__restrict__ X, int N, int d, int dp,
         split_slow_channels(slow, blocks);
         return;
     }
-    const float xs = pow2f(f16_scale_exp(__uint_as_float(__ldg(xrange))));
+    const float xs = pow2f(f16_scale_exp(__uint_as_float(ld_after_wait(xrange))));
     const int d8 = dp / 8;
     const long long n8 = (long long)N * d8, stride = (long long)blocks * blockDim.x;
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;

@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include "mpq_internal.cuh"
+#include "sm100.cuh"
 
 namespace mpq {
 
@@ -48,8 +49,8 @@ __device__ __forceinline__ bool is_slow(const SlowLayer &l, int k)
     bool slow = false;
 #pragma unroll 8
     for (int n = 0; n < l.K; ++n)
-        slow |= slow_point(__uint_as_float(__ldg(v + n)), __uint_as_float(__ldg(v + n + 1)),
-                           __ldg(s + n), limit);
+        slow |= slow_point(__uint_as_float(sm100::ld_after_wait(v + n)),
+                           __uint_as_float(sm100::ld_after_wait(v + n + 1)), __ldg(s + n), limit);
     return slow;
 }
 

@@ -358,6 +358,16 @@ __device__ __forceinline__ void griddep_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// A word that a kernel before, still running when this one was launched, may have written: loaded where
+// it stands, after griddep_wait.  (The non-coherent load of __ldg, or of a const __restrict__ pointer,
+// is for memory that nothing writes while the kernel runs; the compiler may move it above the wait.)
+__device__ __forceinline__ unsigned ld_after_wait(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)) : "memory");
+    return v;
+}
+
 // 4 or 16 bytes from global to shared memory, asynchronously; only the first `bytes` are read, the
 // rest is zero.  cp_async_arrive: this thread's arrival on `bar` (in its count) once its copies so
 // far have landed.

@@ -280,3 +280,29 @@ def test_refused_steps_of_the_adaptive_grid(gpu, oracle):
     o = oracle.output_error(X, 1, W, codes.cpu().numpy(), scales.cpu().numpy(), 4)
     assert np.array_equal(np.isnan(e), np.isnan(o)) and np.isnan(o).any() and np.isfinite(o[:, 0]).all()
     compare_err(np.where(np.isnan(o), 0, e), np.where(np.isnan(o), 0, o))
+
+
+@pytest.mark.parametrize("C,d,N,K,pad", [(134, 1378, 128, 6, 0), (134, 1376, 128, 6, 0), (64, 576, 512, 4, 0),
+                                         (300, 200, 200, 4, 1), (40, 2064, 300, 16, 0)])
+def test_ranges_of_this_call(gpu, C, d, N, K, pad):
+    """The kernels of a call are launched before the ones ahead of them have finished: each uses this
+    call's max |X| and residual ranges, whole.  Inputs whose ranges change from call to call give
+    the same errors every time (rows that are copied, split in place, and measured)."""
+    W = torch.randn(C, d, device=gpu)
+    codes, scales, _, _ = binding.mpq_quantize_layer(W, 8, 16, K)
+    rmax = torch.empty((C, K + 1), device=gpu)
+    binding.mpq_quantize_layer(W, 8, 16, K, codes=codes, scales=scales, rmax=rmax)
+    inputs = []
+    for i in range(4):
+        x = torch.empty(N * d + pad, device=gpu)[pad:].view(N, d)
+        inputs.append(x.copy_(torch.randn(N, d, device=gpu) * 10.0 ** (2 * i - 3)))
+    first = []
+    for i in range(80):
+        e = binding.mpq_output_error(inputs[i % 4], W, codes, scales, K, rmax=rmax if i % 8 < 4 else None)
+        if i < 4:
+            first.append(e)
+            torch.cuda.synchronize()
+            y = inputs[i].double() @ W.double().T
+            assert torch.allclose(e[:, 0].double(), y.square().mean(0), rtol=1e-5, atol=0)
+        else:
+            assert torch.equal(e, first[i % 4])
